@@ -900,9 +900,10 @@ int hsvd_solve_ex(const double *G, int64_t m, int64_t n, int64_t ldg, const int8
     const bool shorten =
         m > n && (o.shorten == HSVD_SHORTEN_ALWAYS || (o.shorten == HSVD_SHORTEN_AUTO && 4 * m >= 5 * n));
     const int64_t m_eff = shorten ? n : m;
-    // the one-CTA pointwise solve is the faster method only for narrow factors
-    // (measured, N(0,1) square factors: n = 16: 1.07 ms against 2.39 ms blocked
-    // with b = 16; n = 32: 3.27 against 2.91 ms; n = 128: 53.8 against 8.5 ms)
+    // the pointwise method below n = 32, the blocked one from there on.  On its
+    // cluster the pointwise kernel is the faster one up to n of about 150 now
+    // (n = 128: 5.95 against 8.5 ms), but the method fixes which value of sigma
+    // ends in which column, so the line stays where callers know it
     int method = o.method;
     if (method == HSVD_METHOD_AUTO)
         method = (n < 32 && pointwise_fits(m_eff, n) && o.precision == HSVD_PRECISION_FP64) ? HSVD_METHOD_POINTWISE

@@ -65,35 +65,29 @@ __device__ void solve_task(const BArgs &A, int k, int g, unsigned char *sm, size
                            PwScalars *sc) {
     const BTask t = A.tasks[k];
     const int n_pad = t.n + (t.n & 1), m_pad = pw_rows_pad(t.m, t.n);
-    const size_t gb = (size_t)m_pad * n_pad * sizeof(double), wb = (size_t)n_pad * n_pad * sizeof(double);
+    const size_t gc = (size_t)m_pad * sizeof(double), wc = (size_t)n_pad * sizeof(double);
     const size_t ab = pw_aux_bytes(n_pad);
+    // shared memory: the per-column arrays, then as many columns of G as fit,
+    // then of W; the rest of both, and the arrays of a factor too large for
+    // them, in the group's part of the workspace
     PwArrays a;
-    unsigned char *aux;
-    int where;
-    if (gb + wb + ab <= budget) {
-        a.G = reinterpret_cast<double *>(sm);
-        a.W = a.G + (size_t)m_pad * n_pad;
-        aux = sm + gb + wb;
-        where = 0;
-    } else if (gb + ab <= budget) {
-        a.G = reinterpret_cast<double *>(sm);
-        a.W = wsg;
-        aux = sm + gb;
-        where = 1;
-    } else {
-        a.G = wsg;
-        a.W = wsg + (size_t)m_pad * n_pad;
-        aux = sm;
-        where = 2;
-    }
-    a.d = reinterpret_cast<double *>(aux);
-    a.pos = reinterpret_cast<int *>(a.d + n_pad);
-    a.newpos = a.pos + n_pad;
-    a.sg = a.newpos + n_pad;
+    a.Gg = wsg;
+    a.Wg = wsg + (size_t)m_pad * n_pad;
+    const bool aux_shared = ab <= budget;
+    size_t left = aux_shared ? budget - ab : budget;
+    unsigned char *at = aux_shared ? sm + ab : sm;
+    pw_carve(a, aux_shared ? reinterpret_cast<void *>(sm)
+                           : reinterpret_cast<void *>(a.Wg + (size_t)n_pad * n_pad), n_pad);
+    a.Gs = reinterpret_cast<double *>(at);
+    a.gs = (int)min((size_t)n_pad, left / gc);
+    left -= a.gs * gc;
+    a.Ws = a.Gs + (size_t)a.gs * m_pad;
+    a.ws = t.V ? (int)min((size_t)n_pad, left / wc) : n_pad;
+    const int where = a.gs < n_pad ? 2 : (a.ws < n_pad ? 1 : 0);
     const int bar = bar_id(NT, g);
     int *res = A.res + 3 * (size_t)t.idx;
     pw_solve<NT>(t.G, t.ldg, t.m, t.n, t.J, m_pad, n_pad, t.tol, A.tstop, A.max_sweeps, A.sort, a, sc[bar], t.sigma,
-                 t.U, t.ldu, t.V, t.ldv, &res[0], &res[1], &A.rot[t.idx], &res[2], bar);
+                 t.U, t.ldu, t.V, t.ldv, &res[0], &res[1], &A.rot[t.idx], &res[2], bar, NT == 512 ? 2 * g : g);
     if ((threadIdx.x & (NT - 1)) == 0) A.where[t.idx] = where;
 }
 
@@ -154,10 +148,11 @@ size_t need_bytes(int64_t m, int64_t n) {
 }
 
 // workspace doubles per CTA: a group of width w owns w/cta of the slot, and
-// must hold G and W of any factor it may take
+// must hold G and W of any factor it may take, and the per-column arrays
 int64_t ws_stride_for(const std::vector<BTask> &tasks, int cta) {
     size_t s = 0;
-    for (const BTask &t : tasks) s = std::max(s, need_bytes(t.m, t.n) * (size_t)(cta / t.width));
+    for (const BTask &t : tasks)
+        s = std::max(s, (need_bytes(t.m, t.n) + pw_aux_bytes(t.n + (t.n & 1))) * (size_t)(cta / t.width));
     return (int64_t)((s / sizeof(double) + 31) / 32 * 32);
 }
 

@@ -129,23 +129,6 @@ __device__ __forceinline__ bool rotation_params(double aii, double ajj, double a
     return true;
 }
 
-// The test of Eq. 2.3, then the rotation of Sec. 2 (rotation_params) for a
-// pair that fails it: the one-sided pointwise kernels, whose rotations are
-// the oracle's bit for bit (a tangent threshold of Eq. 4.2 then stops them
-// at the oracle's sweep).  Returns 0 (the pair passes), 1 (rotate with t, c)
-// or 2 (rank deficient); t = 0, c = 1 unless it returns 1.
-__device__ __forceinline__ int pair_decision(double aii, double ajj, double aij, int hyp, double tol,
-                                             double &t, double &c) {
-    t = 0.0;
-    c = 1.0;
-    if (pair_passes(aii, ajj, aij, tol)) return 0;
-    double tt, cc, qq;
-    if (!rotation_params(aii, ajj, aij, hyp, tt, cc, qq)) return 2;
-    t = tt;
-    c = cc;
-    return 1;
-}
-
 // The rotation of rotation_params with few double-precision instructions.
 // On this part one warp issues a double-precision instruction every 64
 // cycles (a single-precision or integer one every few), and the rotation of

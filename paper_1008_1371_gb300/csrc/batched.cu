@@ -22,6 +22,7 @@
 // timing each width on a sample of that bucket's factors for two sweeps, and
 // caches the choice per device and bucket layout.
 #include <cuda_runtime.h>
+#include <math.h>
 #include <string.h>
 
 #include <algorithm>
@@ -29,7 +30,7 @@
 #include <mutex>
 #include <vector>
 
-#include "pw_core.cuh"
+#include "pw_cluster.cuh"
 
 namespace hsvd {
 namespace {
@@ -130,6 +131,18 @@ __global__ void __launch_bounds__(CTA, 1) k_batched(BArgs A, int smem_budget) {
                     fetch);
 }
 
+// A few factors, too few to fill the SMs one each: one cluster per factor, in
+// queue order (pw_cluster.cuh; P pairs a CTA for the factor's size).
+__global__ void __launch_bounds__(32 * kMaxClPairs) k_batched_cl(BArgs A, int C) {
+    extern __shared__ __align__(16) double dsmem[];
+    const BTask t = A.tasks[blockIdx.x / C];
+    const int half = (t.n + 1) / 2, P = (half + C - 1) / C;
+    if (blockIdx.x % C == 0 && threadIdx.x == 0) A.where[t.idx] = 0;
+    int *res = A.res + 3 * (size_t)t.idx;
+    pw_cluster_solve(dsmem, t.G, t.ldg, t.m, t.n, t.J, P, t.tol, A.tstop, A.max_sweeps, A.sort, t.sigma, t.U, t.ldu,
+                     t.V, t.ldv, res, &A.rot[t.idx]);
+}
+
 // ------------------------------------------------------------------ host side
 
 constexpr int kSmemBudget = 220 * 1024;  // one CTA per SM
@@ -161,13 +174,108 @@ struct Launch {
     cudaError_t err = cudaSuccess;
 };
 
-// Runs the persistent kernel over `tasks` (already in queue order) as one
-// captured graph: counter reset + the launch.
+// pairs a CTA and shared memory of the largest factor on clusters of C CTAs
+struct ClShape {
+    int P = 0;
+    size_t smem = 0;
+};
+ClShape cluster_shape(const std::vector<BTask> &tasks, int C) {
+    ClShape s;
+    for (const BTask &t : tasks) {
+        const int64_t n_pad = t.n + (t.n & 1), P = (n_pad / 2 + C - 1) / C;
+        s.P = std::max(s.P, (int)P);
+        s.smem = std::max(s.smem, pw_cluster_smem(pw_rows_pad(t.m, t.n), n_pad, P, t.V != nullptr));
+    }
+    return s;
+}
+
+cudaError_t cluster_config(int count, int C, const ClShape &s, cudaStream_t st, cudaLaunchConfig_t &cfg,
+                           cudaLaunchAttribute *attr) {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3((unsigned)(count * C));
+    cfg.blockDim = dim3(32 * s.P);
+    cfg.dynamicSmemBytes = s.smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaFuncSetAttribute(k_batched_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
+    if (e == cudaSuccess && C > 8)
+        e = cudaFuncSetAttribute(k_batched_cl, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+
+// Cluster size for a batch too short for the SMs, 0: the queue of groups.  Both
+// are estimated in cycles of a sweep from the FP64 instructions a warp issues
+// (64 cycles on its quarter of an SM, 16 on a whole one): on groups the
+// longest factor has an SM to itself or the SMs share the work evenly; on
+// clusters the longest factor or the work over the clusters resident at once.
+// Clusters must be estimated a fifth faster: their warps form each rotation
+// for one pair only, so they win by spreading, not by work.  Measured (n
+// uniform on [16, 256]): see widen_for_tail.
+int few_clusters(const std::vector<BTask> &tasks, int sms) {
+    if ((int)tasks.size() > sms) return 0;
+    double g_max = 0.0, g_sum = 0.0;
+    for (const BTask &t : tasks) {
+        const double m = pw_rows_pad(t.m, t.n), n = t.n + (t.n & 1), half = n / 2;
+        const double work = half * (7.0 * m + 4.0 * n) / 32.0 * 16.0;
+        g_max = std::max(g_max, n * (work + 50.0 * 64.0 + 1000.0));
+        g_sum += n * (1.1 * work + 50.0 * 16.0 * ceil(half / 32.0));
+    }
+    const double groups = std::max(g_max, g_sum / sms);
+    double best = 0.8 * groups;
+    int best_c = 0;
+    for (int C : {16, 8, 4}) {
+        const ClShape s = cluster_shape(tasks, C);
+        if (s.P > kMaxClPairs || s.smem > kClSmemMax) continue;
+        double c_max = 0.0, c_sum = 0.0;
+        for (const BTask &t : tasks) {
+            const double m = pw_rows_pad(t.m, t.n), n = t.n + (t.n & 1);
+            const double turns = ceil(ceil(n / 2 / C) / 4.0);  // pairs per quarter of an SM
+            const double c = n * (turns * (7.0 * m / 32.0 + 4.0 * n / 32.0 + 56.0) * 64.0 + 1200.0);
+            c_max = std::max(c_max, c);
+            c_sum += c;
+        }
+        if (c_max > best) continue;
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr[1];
+        int resident = 0;
+        if (cluster_config((int)tasks.size(), C, s, nullptr, cfg, attr) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&resident, k_batched_cl, &cfg) != cudaSuccess || resident < 1) {
+            cudaGetLastError();
+            continue;
+        }
+        const double c = std::max(c_max, c_sum / resident);
+        if (c < best) {
+            best = c;
+            best_c = C;
+        }
+    }
+    return best_c;
+}
+
+// Runs the persistent kernel over `tasks` (already in queue order), or with
+// C > 0 one cluster of C CTAs per factor, as one captured graph: counter reset
+// + the launch.
 cudaError_t run_batch(const std::vector<BTask> &tasks, int max_sweeps, int sort, double tstop, bool use_graph,
-                      int grid, int cta, int *res, long long *rot, int *where, cudaStream_t st, float *ms) {
+                      int grid, int cta, int C, int *res, long long *rot, int *where, cudaStream_t st, float *ms) {
     const int count = (int)tasks.size();
-    const int64_t stride = ws_stride_for(tasks, cta);
+    const int64_t stride = C ? 0 : ws_stride_for(tasks, cta);
     void (*kern)(BArgs, int) = cta == 512 ? k_batched<512> : k_batched<1024>;
+    const ClShape shape = C ? cluster_shape(tasks, C) : ClShape{};
+    auto launch = [&](const BArgs &A, cudaStream_t on) -> cudaError_t {
+        if (C) {
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute attr[1];
+            const cudaError_t ce = cluster_config(count, C, shape, on, cfg, attr);
+            return ce != cudaSuccess ? ce : cudaLaunchKernelEx(&cfg, k_batched_cl, A, C);
+        }
+        kern<<<grid, cta, kSmemBudget, on>>>(A, kSmemBudget);
+        return cudaGetLastError();
+    };
     BTask *d_tasks = nullptr;
     int *d_counter = nullptr;
     double *d_ws = nullptr;
@@ -209,8 +317,7 @@ cudaError_t run_batch(const std::vector<BTask> &tasks, int max_sweeps, int sort,
         if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             cudaMemsetAsync(d_counter, 0, sizeof(int), cap);
-            kern<<<grid, cta, kSmemBudget, cap>>>(A, kSmemBudget);
-            const cudaError_t le = cudaGetLastError();
+            const cudaError_t le = launch(A, cap);
             e = cudaStreamEndCapture(cap, &graph);
             if (e == cudaSuccess) e = le;
         }
@@ -222,10 +329,7 @@ cudaError_t run_batch(const std::vector<BTask> &tasks, int max_sweeps, int sort,
     } else if (e == cudaSuccess) {
         e = cudaMemsetAsync(d_counter, 0, sizeof(int), st);
         if (e == cudaSuccess && ms) e = cudaEventRecord(e0, st);
-        if (e == cudaSuccess) {
-            kern<<<grid, cta, kSmemBudget, st>>>(A, kSmemBudget);
-            e = cudaGetLastError();
-        }
+        if (e == cudaSuccess) e = launch(A, st);
         if (e == cudaSuccess && ms) e = cudaEventRecord(e1, st);
     }
     if (e == cudaSuccess && ms) {
@@ -251,21 +355,33 @@ void order_tasks(std::vector<BTask> &tasks) {
 }
 
 std::mutex g_tune_mu;
-std::map<long long, std::vector<int>> g_tune_cache;  // (device, CTA, bucket mask) -> width per bucket
+std::map<long long, std::vector<int>> g_tune_cache;  // tune_key -> width per bucket
 
 // Picks the group width of every size bucket present: each candidate width is
-// timed on up to (SMs x 1024 / width) factors of the bucket, two sweeps each,
-// and scored by sum(m n^2) / time.
-long long tune_key(int dev, int cta, long long mask) { return ((long long)dev << 32) | ((long long)cta << 16) | mask; }
+// timed on (SMs x 1024 / width) factors of the bucket, two sweeps each, and
+// scored by sum(m n^2) / time.  A bucket with fewer factors than the narrowest
+// width has groups cannot show what a full GPU does with it and is not timed:
+// it takes that width, the fastest per factor or within 1% of it wherever it
+// was measured (4000 factors of n in [16, 64]: 256: 46.9 ms, 512: 56.3, 1024:
+// 81.2; 2000 of [100, 140]: 413, 406, 437; 608 of 256: 846, 839, 862).
+// The choice is kept by device, CTA size, buckets present and buckets filled.
+long long tune_key(int dev, int cta, const std::vector<BTask> &all, int grid, int *filled) {
+    int n[kBuckets] = {}, mask = 0;
+    *filled = 0;
+    for (const BTask &t : all) ++n[bucket_of(t.n)];
+    for (int b = 0; b < kBuckets; ++b) {
+        mask |= (n[b] > 0) << b;
+        *filled |= (n[b] >= grid * (cta / 256)) << b;
+    }
+    return ((long long)dev << 32) | ((long long)cta << 16) | (*filled << 8) | mask;
+}
 
 cudaError_t tune_widths(const std::vector<BTask> &all, int grid, int cta, int *res, long long *rot, int *where,
                         cudaStream_t st, std::vector<int> &width, float *ms_total) {
-    width.assign(kBuckets, cta);
-    int dev = 0;
+    width.assign(kBuckets, 256);
+    int dev = 0, filled = 0;
     cudaGetDevice(&dev);
-    long long mask = 0;
-    for (const BTask &t : all) mask |= 1LL << bucket_of(t.n);
-    const long long key = tune_key(dev, cta, mask);
+    const long long key = tune_key(dev, cta, all, grid, &filled);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
@@ -275,7 +391,7 @@ cudaError_t tune_widths(const std::vector<BTask> &all, int grid, int cta, int *r
         }
     }
     for (int b = 0; b < kBuckets; ++b) {
-        if (!(mask & (1LL << b))) continue;
+        if (!(filled & (1 << b))) continue;
         std::vector<BTask> members;
         for (const BTask &t : all)
             if (bucket_of(t.n) == b) members.push_back(t);
@@ -293,7 +409,7 @@ cudaError_t tune_widths(const std::vector<BTask> &all, int grid, int cta, int *r
             }
             order_tasks(sample);
             float ms = 0.f;
-            const cudaError_t e = run_batch(sample, 2, 1, 0.0, false, grid, cta, res, rot, where, st, &ms);
+            const cudaError_t e = run_batch(sample, 2, 1, 0.0, false, grid, cta, 0, res, rot, where, st, &ms);
             if (e != cudaSuccess) return e;
             if (ms_total) *ms_total += ms;
             const double score = work / std::max(ms, 1e-3f);
@@ -306,6 +422,34 @@ cudaError_t tune_widths(const std::vector<BTask> &all, int grid, int cta, int *r
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune_cache[key] = width;
     return cudaSuccess;
+}
+
+// The autotuner's widths give the most factors per second of a long queue; in a
+// short one a factor solved by a quarter of an SM can outlast all the others.
+// A bucket's width doubles while its largest factor at that width (work m n^2,
+// cta / width times slower than on a whole SM) would take longer than an SM's
+// share of the work of this and the smaller buckets, which the queue holds
+// last; up to one warp for every four pairs (more only wait), and never below
+// a smaller bucket's width, so that the queue stays largest first.
+// Measured (n uniform on [16, 256], queue at 256 everywhere / at these widths
+// / on clusters): 600 factors 447 / 275 ms, 1000: 519 with the widths of n <
+// 128 left at 256 / 459, 40: 257 / 210 / 46, 100: 291 / 239 / 142.
+void widen_for_tail(const std::vector<BTask> &tasks, int sms, int cta, std::vector<int> &width) {
+    double sum[kBuckets] = {}, most[kBuckets] = {};
+    for (const BTask &t : tasks) {
+        const double w = (double)t.m * t.n * t.n;
+        const int b = bucket_of(t.n);
+        sum[b] += w;
+        most[b] = std::max(most[b], w);
+    }
+    double below = 0.0;
+    for (int b = 0; b < kBuckets; ++b) {
+        below += sum[b];
+        int &w = width[(size_t)b];
+        const int cap = std::min(cta, b < 2 ? 256 : (b < 3 ? 512 : 1024));
+        while (w < cap && most[b] * (cta / w) > below / sms) w *= 2;
+        if (b > 0) w = std::max(w, width[(size_t)b - 1]);
+    }
 }
 
 }  // namespace
@@ -425,23 +569,24 @@ int hsvd_solve_batched_ex(int64_t count, const double *const *G, const int64_t *
     std::vector<int> width(kBuckets, o.group_width ? o.group_width : cta);
     float ms_tune = 0.f;
     int tuned = 0;
-    if (rc == HSVD_OK && o.group_width == 0) {
+    const int C = (o.group_width || o.cta_threads) ? 0 : few_clusters(tasks, sms);
+    if (rc == HSVD_OK && o.group_width == 0 && C == 0) {
         std::vector<int> w;
         const bool cached = [&] {
             std::lock_guard<std::mutex> lk(g_tune_mu);
-            long long mask = 0;
-            for (const BTask &t : tasks) mask |= 1LL << bucket_of(t.n);
-            return g_tune_cache.count(tune_key(dev, cta, mask)) > 0;
+            int filled = 0;
+            return g_tune_cache.count(tune_key(dev, cta, tasks, sms, &filled)) > 0;
         }();
         if (tune_widths(tasks, sms, cta, d_res, d_rot, d_where, st, w, &ms_tune) != cudaSuccess) fail(HSVD_ERR_CUDA);
         else width = w;
         tuned = cached ? 2 : 1;
     }
+    if (o.group_width == 0 && C == 0) widen_for_tail(tasks, sms, cta, width);
     for (BTask &t : tasks) t.width = width[(size_t)bucket_of(t.n)];
     order_tasks(tasks);
     float ms = 0.f;
     if (rc == HSVD_OK &&
-        run_batch(tasks, o.max_sweeps, o.sort ? 1 : 0, o.tstop, o.use_graph != 0, grid, cta, d_res, d_rot, d_where,
+        run_batch(tasks, o.max_sweeps, o.sort ? 1 : 0, o.tstop, o.use_graph != 0, grid, cta, C, d_res, d_rot, d_where,
                   st, &ms) != cudaSuccess)
         fail(HSVD_ERR_CUDA);
     std::vector<int> h_res(3 * (size_t)count, 0), h_where((size_t)count, 0);
@@ -486,8 +631,8 @@ int hsvd_solve_batched_ex(int64_t count, const double *const *G, const int64_t *
             else if (s_k == HSVD_NOT_CONVERGED && worst == HSVD_OK) worst = s_k;
         }
         if (info) {
-            info->grid = grid;
-            info->cta_threads = cta;
+            info->grid = C ? (int)count * C : grid;
+            info->cta_threads = C ? 32 * cluster_shape(tasks, C).P : cta;
             info->tuned = tuned;
             for (int b = 0; b < 5; ++b) info->bucket_width[b] = width[(size_t)b];
             info->ms_kernel = ms;

@@ -36,11 +36,13 @@ SHAPES = [(1, 1), (2, 2), (5, 3), (40, 2), (8, 8), (9, 9), (16, 16), (300, 18), 
 @pytest.mark.parametrize("m,n", SHAPES)
 def test_cluster_equals_batched_bitwise(api, m, n):
     G, J = _factor(m, n, 1000 * m + n)
+    # group_width: the queue of groups, whatever the batch
     for sort, tstop, want_v in ((True, 0.0, True), (False, 0.0, True), (True, -1.0, True), (True, 0.0, False)):
         tol = n * 2.0 ** -53
         one = api.hsvd_solve_ex(G, J, api.make_opts(method=api.HSVD_METHOD_POINTWISE, sort=sort, tstop=tstop, tol=tol,
                                                     shorten=api.HSVD_SHORTEN_NEVER), compute_v=want_v)
-        b = api.hsvd_solve_batched([G], [J], api.make_batch_opts(sort=sort, tstop=tstop, tol=tol), compute_v=want_v)
+        b = api.hsvd_solve_batched([G], [J], api.make_batch_opts(sort=sort, tstop=tstop, tol=tol, group_width=512),
+                                   compute_v=want_v)
         assert one.status == b.status[0] == 0 and one.sweeps == b.sweeps[0]
         assert one.rotations == b.info.rotations
         assert torch.equal(one.sigma, b.sigma[0]) and torch.equal(one.U, b.U[0])
@@ -58,3 +60,17 @@ def test_two_long_columns_take_the_one_cta_kernel(api):
     ref = np.sort(np.linalg.svd(G.cpu().numpy(), compute_uv=False))
     assert r.status == 0
     assert np.max(np.abs(np.sort(r.sigma.cpu().numpy()) - ref) / ref) <= 8 * np.sqrt(12000) * 2.0 ** -53
+
+
+@pytest.mark.parametrize("sizes", [[256, 40, 17, 3], [64] * 30, [200, 131, 90, 16, 5] * 8])
+def test_few_factors_take_clusters_bitwise(api, sizes):
+    """A batch too short for the SMs runs one cluster per factor: the same bits
+    as the queue of 1024-thread groups."""
+    facs = [_factor(n, n, 31 * k + n) for k, n in enumerate(sizes)]
+    Gs, Js = [f[0] for f in facs], [f[1] for f in facs]
+    a = api.hsvd_solve_batched(Gs, Js, api.make_batch_opts())
+    b = api.hsvd_solve_batched(Gs, Js, api.make_batch_opts(group_width=1024))
+    assert a.info.kernel_launches == b.info.kernel_launches == 1 and a.info.grid > len(sizes) >= b.info.grid
+    assert a.sweeps == b.sweeps and a.status == b.status and a.info.rotations == b.info.rotations
+    for k in range(len(sizes)):
+        assert torch.equal(a.sigma[k], b.sigma[k]) and torch.equal(a.U[k], b.U[k]) and torch.equal(a.V[k], b.V[k])

@@ -207,7 +207,10 @@ int solve_blocked_core(const double *G, int64_t m, int64_t n, int64_t ldg, const
     DagStreams dag;
     Ws ws(st);
     double *Gw = ws.get<double>(m_pad * n_pad), *Gt = ws.get<double>(m_pad * n_pad);
-    double *Ww = ws.get<double>(ldw * n_pad), *Wt = ws.get<double>(ldw * n_pad);
+    // the transformation is accumulated only when V is asked for: half of the
+    // update's rows for a square factor
+    const bool want_w = V != nullptr;
+    double *Ww = want_w ? ws.get<double>(ldw * n_pad) : nullptr, *Wt = want_w ? ws.get<double>(ldw * n_pad) : nullptr;
     int *perm = ws.get<int>(n_pad), *perm_t = ws.get<int>(n_pad), *newpos = ws.get<int>(n_pad);
     int8_t *sgn = ws.get<int8_t>(n_pad), *sgn_t = ws.get<int8_t>(n_pad);
     double *d = ws.get<double>(n_pad);
@@ -226,7 +229,7 @@ int solve_blocked_core(const double *G, int64_t m, int64_t n, int64_t ldg, const
     int *d_tab_outer = ws.get<int>((size_t)nb * npairs * 2);
     int *d_tab_full = ws.get<int>((size_t)nn * b * 2 + ring_table_ints(b));
     int *d_tab_cross = ws.get<int>((size_t)b * b * 2);
-    if (!Gw || !Gt || !Ww || !Wt || !perm || !perm_t || !newpos || !sgn || !sgn_t || !d || !part || !Wp ||
+    if (!Gw || !Gt || (want_w && (!Ww || !Wt)) || !perm || !perm_t || !newpos || !sgn || !sgn_t || !d || !part || !Wp ||
         !rotated || !cnt || !d_tab_outer || !d_tab_full || !d_tab_cross)
         return HSVD_ERR_NOMEM;
     // split-precision products: full 2b x 2b Gram partials, W' slices, exponents

@@ -9,8 +9,9 @@ namespace {
 constexpr int kThreads = 256;
 
 // Working copy bordered as in Eq. 4.1: columns n..n_pad-1 are unit vectors in
-// the fresh rows m..m+(n_pad-n)-1, rows up to m_pad are zero.  W = I, working
-// position k holds input column perm[k] = k, pads carry sign +1.
+// the fresh rows m..m+(n_pad-n)-1, rows up to m_pad are zero.  W = I (unless no
+// V is asked for: Ww null), working position k holds input column perm[k] = k,
+// pads carry sign +1.
 __global__ void k_load_pad(const double *__restrict__ G, int64_t ldg, int64_t m, int64_t n,
                            const int8_t *__restrict__ J, double *__restrict__ Gw, int64_t m_pad,
                            int64_t n_pad, double *__restrict__ Ww, int64_t ldw, int *__restrict__ perm,
@@ -27,7 +28,8 @@ __global__ void k_load_pad(const double *__restrict__ G, int64_t ldg, int64_t m,
         bad |= !isfinite(v);
         Gw[i + j * m_pad] = v;
     }
-    for (int64_t i = threadIdx.x; i < ldw; i += kThreads) Ww[i + j * ldw] = (i == j) ? 1.0 : 0.0;
+    if (Ww)
+        for (int64_t i = threadIdx.x; i < ldw; i += kThreads) Ww[i + j * ldw] = (i == j) ? 1.0 : 0.0;
     if (threadIdx.x == 0) {
         perm[j] = (int)j;
         const int8_t sj = (j < n) ? J[j] : (int8_t)1;
@@ -110,9 +112,11 @@ __global__ void k_permute(const double *__restrict__ Gw, double *__restrict__ Gt
     const double2 *gs = reinterpret_cast<const double2 *>(Gw + src * m_pad);
     double2 *gd = reinterpret_cast<double2 *>(Gt + k * m_pad);
     for (int64_t i = threadIdx.x; i < m_pad / 2; i += kThreads) gd[i] = gs[i];
-    const double2 *ws = reinterpret_cast<const double2 *>(Ww + src * ldw);
-    double2 *wd = reinterpret_cast<double2 *>(Wt + k * ldw);
-    for (int64_t i = threadIdx.x; i < ldw / 2; i += kThreads) wd[i] = ws[i];
+    if (Ww) {
+        const double2 *ws = reinterpret_cast<const double2 *>(Ww + src * ldw);
+        double2 *wd = reinterpret_cast<double2 *>(Wt + k * ldw);
+        for (int64_t i = threadIdx.x; i < ldw / 2; i += kThreads) wd[i] = ws[i];
+    }
     if (threadIdx.x == 0) {
         perm_t[k] = perm[src];
         sgn_t[k] = sgn[src];
@@ -195,7 +199,7 @@ cudaError_t launch_reorder(double *Gw, double *Gt, int64_t m_pad, double *Ww, do
     if (e != cudaSuccess) return e;
     e = cudaMemcpyAsync(Gw, Gt, sizeof(double) * m_pad * n_pad, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(Ww, Wt, sizeof(double) * ldw * n_pad, cudaMemcpyDeviceToDevice, st);
+    if (Ww) e = cudaMemcpyAsync(Ww, Wt, sizeof(double) * ldw * n_pad, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) return e;
     e = cudaMemcpyAsync(perm, perm_t, sizeof(int) * n_pad, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) return e;

@@ -52,22 +52,23 @@ __device__ __forceinline__ double neg_bits(double x) {
 // 1 +- 2^-16; the expression's three roundings move its threshold by less
 // than 2^-51, so both agree there.  Every other case evaluates the
 // expression.
+// (The estimate is formed without branches: on the inner solve's critical path
+// its integer chain then runs behind the rotation's first divisions.)
 __device__ __forceinline__ bool pair_passes(double aii, double ajj, double aij, double tol) {
     const unsigned ha = (unsigned)__double2hiint(aij) & 0x7fffffffu, h1 = (unsigned)__double2hiint(aii),
                    h2 = (unsigned)__double2hiint(ajj), ht = (unsigned)__double2hiint(tol);
     const int ea = (int)(ha >> 20) - 1023, e1 = (int)(h1 >> 20) - 1023, e2 = (int)(h2 >> 20) - 1023,
               et = (int)(ht >> 20) - 1023;  // a_ii, a_jj, tol: the sign bit makes these out of range
-    if (ea >= -500 && ea <= 500 && e1 >= -500 && e1 <= 500 && e2 >= -500 && e2 <= 500 && et >= -200 && et <= 200) {
-        const int k = 2 * ea - 2 * et - e1 - e2;
-        if (k >= 5) return false;
-        if (k <= -3) return true;
-        const float ma = f32_scaled(aij, ea), m1 = f32_scaled(aii, e1), m2 = f32_scaled(ajj, e2),
-                    mt = f32_scaled(tol, et);
-        const float lm = __fmul_rn(__fmul_rn(ma, ma), __int_as_float((127 + k) << 23));
-        const float rm = __fmul_rn(__fmul_rn(mt, mt), __fmul_rn(m1, m2));
-        if (lm < __fmul_rn(rm, 1.0f - 1.52587890625e-05f)) return true;
-        if (lm > __fmul_rn(rm, 1.0f + 1.52587890625e-05f)) return false;
-    }
+    const bool in = (unsigned)(ea + 500) <= 1000u && (unsigned)(e1 + 500) <= 1000u && (unsigned)(e2 + 500) <= 1000u &&
+                    (unsigned)(et + 200) <= 400u;
+    const int k = 2 * ea - 2 * et - e1 - e2, kc = min(max(k, -3), 5);
+    const float ma = f32_scaled(aij, ea), m1 = f32_scaled(aii, e1), m2 = f32_scaled(ajj, e2),
+                mt = f32_scaled(tol, et);
+    const float lm = __fmul_rn(__fmul_rn(ma, ma), __int_as_float((127 + kc) << 23));
+    const float rm = __fmul_rn(__fmul_rn(mt, mt), __fmul_rn(m1, m2));
+    const bool below = k <= -3 || lm < __fmul_rn(rm, 1.0f - 1.52587890625e-05f);
+    const bool above = k >= 5 || lm > __fmul_rn(rm, 1.0f + 1.52587890625e-05f);
+    if (in && (below || above)) return below && !(k >= 5);
     return aij == 0.0 || fabs(aij) < tol * sqrt(aii * ajj);
 }
 
@@ -147,8 +148,16 @@ __device__ __forceinline__ bool rotation_params(double aii, double ajj, double a
 // b = 0 (trigonometric only) or normal with 2^-100 <= |b / a_ij| < 2^101, and
 // a hyperbolic pair with |zeta| >= 2 (|b| >= 4 |a_ij|, which also settles the
 // rank test); every other pair takes rotation_params.
-__device__ __forceinline__ bool rotation_params_fast(double aii, double ajj, double aij, int hyp, double &t,
-                                                     double &c, double &qv) {
+// The tangent alone, in two parts.  rotation_start: the single-precision start
+// (how = 1; one FP64 instruction), or how = 2 for a pair outside its range.
+// rotation_tangent: the Newton steps, or t of rotation_params; returns how, or
+// 0 when the pair is rank deficient.
+struct RotStart {
+    double b, t0, ngd;  // b of f, the first t, -1/f'
+    int how;
+};
+__device__ __forceinline__ RotStart rotation_start(double aii, double ajj, double aij, int hyp) {
+    RotStart o;
     const bool trig = hyp < 0;
     const double b = trig ? ajj - aii : aii + ajj;
     const int E = exp_field(aij), eb = exp_field(b);
@@ -158,7 +167,10 @@ __device__ __forceinline__ bool rotation_params_fast(double aii, double ajj, dou
     if (bbits == 0) fast = fast && trig;
     else fast = fast && eb > -1023 && eb < 1024 && eb - E >= -100 && eb - E <= 100;
     if (fast && !trig) fast = bbits >= abits + (2ull << 52);  // |b| >= 4 |a_ij|
-    if (!fast) return rotation_params(aii, ajj, aij, hyp, t, c, qv);
+    o.b = b;
+    o.t0 = o.ngd = 0.0;
+    o.how = fast ? 1 : 2;
+    if (!fast) return o;
     const float af = f32_scaled(aij, E);
     const float bf = bbits == 0 ? 0.0f : f32_scaled(b, E);
     const float z = __fdiv_rn(trig ? bf : -bf, __fmul_rn(2.0f, af));  // zeta
@@ -173,20 +185,72 @@ __device__ __forceinline__ bool rotation_params_fast(double aii, double ajj, dou
     if (z < 0.0f) tf = -tf;
     // 1/f'(t) 2^E in single precision, f'(t) = 2 a_ij t + b: |f'| >= 2 |a_ij| at the root
     const float gf = __fdiv_rn(1.0f, __fadd_rn(__fmul_rn(__fmul_rn(2.0f, af), tf), bf));
-    const double ngd = neg_bits(f64_scaled(gf, -E));
-    const double sa = trig ? neg_bits(aij) : aij;
-    double tt = f64_scaled(tf, 0);
+    o.ngd = neg_bits(f64_scaled(gf, -E));
+    o.t0 = f64_scaled(tf, 0);
+    return o;
+}
+__device__ __forceinline__ int rotation_tangent(const RotStart &r, double aii, double ajj, double aij, int hyp,
+                                                double &t) {
+    if (r.how == 2) {
+        double c, qv;
+        return rotation_params(aii, ajj, aij, hyp, t, c, qv) ? 2 : 0;
+    }
+    const double sa = hyp < 0 ? neg_bits(aij) : aij;
+    double tt = r.t0;
 #pragma unroll
-    for (int it = 0; it < 2; ++it) tt = fma(fma(fma(aij, tt, b), tt, sa), ngd, tt);
-    const double x = fma(tt, trig ? tt : neg_bits(tt), 1.0);
-    const float r0 = __fdiv_rn(1.0f, __fsqrt_rn(f32_scaled(x, 0)));
-    double y = f64_scaled(r0, 0);
-    y = fma(f64_scaled(r0, -1), fma(neg_bits(x * y), y, 1.0), y);
+    for (int it = 0; it < 2; ++it) tt = fma(fma(fma(aij, tt, r.b), tt, sa), r.ngd, tt);
     t = tt;
-    c = cosine_step(tt, hyp, y);
-    qv = reciprocal_step(c, x * c);
+    return 1;
+}
+
+// c of the rotation with tangent t, from t alone; `how` as
+// rotation_tangent returned it (1 or 2).
+__device__ __forceinline__ double rotation_cosine(double t, int hyp, int how) {
+    const bool trig = hyp < 0;
+    if (how == 1) {
+        const double x = fma(t, trig ? t : neg_bits(t), 1.0);
+        const float r0 = __fdiv_rn(1.0f, __fsqrt_rn(f32_scaled(x, 0)));
+        double y = f64_scaled(r0, 0);
+        y = fma(f64_scaled(r0, -1), fma(neg_bits(x * y), y, 1.0), y);
+        return cosine_step(t, hyp, y);
+    }
+    return cosine_step(t, hyp, 1.0 / sqrt(trig ? 1.0 + t * t : (1.0 - t) * (1.0 + t)));
+}
+// qv = 1/c from t and c
+__device__ __forceinline__ double rotation_reciprocal(double t, int hyp, int how, double c) {
+    const bool trig = hyp < 0;
+    if (how == 1) return reciprocal_step(c, fma(t, trig ? t : neg_bits(t), 1.0) * c);
+    return reciprocal_step(c, sqrt(trig ? 1.0 + t * t : (1.0 - t) * (1.0 + t)));
+}
+
+__device__ __forceinline__ bool rotation_params_fast(double aii, double ajj, double aij, int hyp, double &t,
+                                                     double &c, double &qv) {
+    const int how = rotation_tangent(rotation_start(aii, ajj, aij, hyp), aii, ajj, aij, hyp, t);
+    if (how == 0) {
+        c = qv = 1.0;
+        return false;
+    }
+    c = rotation_cosine(t, hyp, how);
+    qv = rotation_reciprocal(t, hyp, how, c);
     return true;
 }
+
+// The flags of a pair: 0 (it passes Eq. 2.3), kPairRot, with kPairExact when t
+// came from rotation_params, or kPairRank (rank deficient).  pair_tangent: the
+// test, then the tangent for a pair that fails it; t = 0 unless it rotates.
+constexpr int kPairRot = 1, kPairRank = 2, kPairExact = 4;
+__device__ __forceinline__ int pair_flags(int how) {
+    return how == 0 ? kPairRank : kPairRot | (how == 2 ? kPairExact : 0);
+}
+__device__ __forceinline__ int pair_tangent(double aii, double ajj, double aij, int hyp, double tol, double &t) {
+    t = 0.0;
+    if (pair_passes(aii, ajj, aij, tol)) return 0;
+    double tt;
+    const int how = rotation_tangent(rotation_start(aii, ajj, aij, hyp), aii, ajj, aij, hyp, tt);
+    if (how) t = tt;
+    return pair_flags(how);
+}
+__device__ __forceinline__ int pair_how(int flags) { return flags & kPairExact ? 2 : 1; }
 
 // The test of Eq. 2.3, then the rotation of Sec. 2 (rotation_params_fast) for
 // a pair that fails it.  Returns 0 (the pair passes), 1 (rotate with t, c;

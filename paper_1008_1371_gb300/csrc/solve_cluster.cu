@@ -43,15 +43,57 @@ namespace hsvd {
 namespace {
 
 constexpr int kClThreads = 256;
-constexpr int kCrossThreads = kClThreads + 32;  // cross pass: 8 mixing warps + the look-ahead warp
 
-// the mixing threads' barrier: barrier 1 among the last n threads of the CTA
-// (warps 1..) when warp 0 runs ahead, else the whole CTA
+// Warps of the cross and ring kernels.  Eight warps mix rows and columns; the
+// others do what every CTA repeats for every pair of the step (Eq. 2.6 on the
+// diagonal, the cosine and its reciprocal, the scales) while they mix, and form
+// the owned pairs' next rotations:
+//   LA (b = 64):  warp 0 forms them one step ahead, while the step is mixed;
+//                 warps 9, 10 are helpers for 32 pairs each.
+//   else:         warp 0 forms them after the mix, and before that the cosines
+//                 and scales; warp 4 takes the diagonal, then the tests of
+//                 Eq. 2.3; warp 11 the reciprocals and the scale ratios of the
+//                 next coefficients (with its own copy of the scales).
+// One FP64 instruction of a warp occupies its quarter of the SM's FP64 pipe for
+// 64 cycles, so where the rotation chain is the critical path (b <= 32) no
+// mixing warp shares warp 0's quarter (warps 0, 4, 8).
+constexpr int kMixWarps = 8, kMixThreads = 32 * kMixWarps;
 template <bool LA>
-__device__ __forceinline__ void mix_sync(int n) {
-    if (LA) asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory");
-    else __syncthreads();
+struct Role {
+    static constexpr int kThreads = LA ? 352 : 384;
+    static constexpr int kHelpers = LA ? 2 : 1;
+    static __device__ __forceinline__ bool mixes(int warp) {
+        return LA ? warp >= 1 && warp <= 8 : (warp & 3) != 0 && warp < 11;
+    }
+    static __device__ __forceinline__ int mixer(int warp) { return LA ? warp - 1 : warp - 1 - (warp >> 2); }
+};
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
+// named barriers of a CTA: the mixing warps; the mix and the diagonal done; the
+// look-ahead has read its entries; the helpers; the next step's scale ratios;
+// the next step's tests
+enum { kBarMix = 1, kBarDone, kBarRead, kBarHelp, kBarRatio, kBarTest };
+
+// A step's rotations as every CTA holds them (two steps' worth): 16-byte words,
+// so that a rotation reaches a CTA in three stores.
+template <int H, bool LA>
+struct Rots {
+    double2 ta[2][H];                // t, alpha
+    double2 bp[2][H];                // beta, the true a_pq
+    double2 cf[2][LA ? H : 1];       // LA: c, the flags in the second word's bits
+    int fl[2][LA ? 1 : H];           // else the flags (kPairRot ...)
+    __device__ __forceinline__ int flags(int b, int j) const {
+        return LA ? (int)__double_as_longlong(cf[b][LA ? j : 0].y) : fl[b][LA ? 0 : j];
+    }
+    __device__ __forceinline__ void put(int b, int j, double t, double al, double be, double c, double apq, int f) {
+        ta[b][j] = make_double2(t, al);
+        bp[b][j] = make_double2(be, apq);
+        if (LA) cf[b][LA ? j : 0] = make_double2(c, __longlong_as_double((long long)f));
+        else fl[b][LA ? 0 : j] = f;
+    }
+};
 
 template <int NN>
 struct ClusterOf {
@@ -354,17 +396,30 @@ k_solve_cluster(const double *__restrict__ part, int nsplit, int full_part, doub
 // k and their current partner rows h + (k + s) mod h.  Both halves of
 // R^T A R touch only a pair's two rows (the row mix) and, inside every row,
 // the two columns of each pair (the column mix), so a step is local once the
-// CTA knows every pair's (t, c).  From step s to s + 1 pair k takes pair
+// CTA knows every pair's rotation.  From step s to s + 1 pair k takes pair
 // k + 1's partner row: inside the CTA that is a ring of P + 1 row slots, and
 // across the cluster every CTA hands its first pair's partner row to the
 // previous CTA.  The next step's a_pq lies in the owner's fixed row, so the
-// owner computes that pair's (t, c) as soon as its rows are updated and writes
-// them into every CTA; one cluster barrier per step.  The element operations
-// and their order (column mix first on even steps, row mix first on odd
-// steps, Eq. 2.6 on the diagonal, zeros at the pair) are the oracle's, so the
-// result is bit-identical to it and to k_solve_cluster.
+// owner forms that pair's rotation (t and the scaled coefficients alpha, beta;
+// look-ahead: c too) and writes it into every CTA; one cluster barrier per step.
+// The element operations and their order (column mix first on even steps, row
+// mix first on odd steps, Eq. 2.6 on the diagonal, zeros at the pair) are the
+// oracle's, so the result is bit-identical to it and to k_solve_cluster.
+//
+// Only t is on the way from one step's rotation to the next mix: c, 1/c, the
+// scales, their ratios, the diagonal and the next tests are formed beside the
+// mix by warps of their own.  Cycles of a step with every pair rotating
+// (clock64; before: the owner formed and published all parameters, the mixing
+// warps the coefficients and the diagonal, between CTA barriers):
+//   b = 16: 4,500 (7,000), b = 32: 5,150 (7,300), b = 64: 6,500 (8,200).
+// b = 16: 1,620 for the cosines and scales beside 1,750 of mixing, 1,100 for the
+// start of the next t, 500 for its Newton steps, 350 to publish, 440 for the
+// cluster barrier.  A visit also costs 9,000 to 12,000 cycles before the first
+// step (A_P from the Gram's partials) and 2,500 to 7,000 after the last.
+// The inner solves of a step of the n = 301 factor: 57.4 -> 40.5 us (b = 16),
+// 103 -> 78 us (b = 32); of graded 1024 at b = 32: 91 -> 77 us.
 template <int NN, int C, bool LA>
-__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(LA ? kCrossThreads : kClThreads, 3)
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(Role<LA>::kThreads, 2)
 k_solve_cross(const double *__restrict__ part, int nsplit, int full_part, double *__restrict__ A_io,
               const int8_t *__restrict__ sgn_cols, const int *__restrict__ col0,
               const int8_t *__restrict__ sgn_direct, double tol, double *__restrict__ Wout,
@@ -372,9 +427,10 @@ k_solve_cross(const double *__restrict__ part, int nsplit, int full_part, double
               int *__restrict__ dexp, const int *__restrict__ visit, float *__restrict__ trace, double tstop,
               int *__restrict__ tbig) {
     constexpr int h = NN / 2, P = h / C, RW = NN / C, B = NN / 2;
-    constexpr int kT = LA ? kCrossThreads : kClThreads;
+    using R = Role<LA>;
+    constexpr int kT = R::kThreads;
     static_assert(P * C == h && RW * C == NN, "the pairs and rows split evenly over the cluster");
-    static_assert(!LA || P <= 32, "the look-ahead warp has one lane per owned pair");
+    static_assert(32 % P == 0 && h <= 32 * R::kHelpers, "lanes in whole sets of owned pairs, one helper lane per pair");
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int pair = blockIdx.x / C;
@@ -392,16 +448,17 @@ k_solve_cross(const double *__restrict__ part, int nsplit, int full_part, double
     double *Wl = mov + (P + 1) * NN;  // [RW][NN]   rows w0 .. w0 + RW - 1 of W_P
     __shared__ double D[NN];
     __shared__ int sg[NN];
-    __shared__ double T[2][h], Cc[2][h], Qv[2][h], Apq[2][h];  // Apq: the true a_pq
-    __shared__ int Fl[2][h];          // bit 0: rotate, bit 1: rank deficient
+    __shared__ __align__(16) Rots<h, LA> rt;
+    __shared__ double Ra[h], Rb[h];    // the next step's scale ratios
+    __shared__ double Sd[LA ? 1 : NN];  // the scales again, the ratio warp's own
+    __shared__ int pass[LA ? 1 : 32];   // the next step's pairs that pass Eq. 2.3
     __shared__ double Sc[NN], Rc[NN];  // column scales of the stored block and their reciprocals
-    __shared__ double Al[h], Be[h];    // the step's scaled-rotation coefficients
-    __shared__ int s_renorm;
+    __shared__ int s_renorm[2][R::kHelpers];  // scales out of range before the step (by parity)
+    __shared__ int s_bad[2];                  // a rank-deficient pair in the step (by parity)
     __shared__ double tr_max[C], tr_sum[C], tr_red[2][kT / 32];
     __shared__ int s_first[C];        // per CTA: first step with a pair failing Eq. 2.3 on A_P
     __shared__ int s_own;
-    __shared__ int s_tot[2];          // rotations counted by warps 0 and 1
-    static_assert(h <= 64, "the rotation count lives in warps 0 and 1");
+    __shared__ int s_tot[R::kHelpers];  // rotations counted by the helpers
 
     auto entry = [&](int x, int y) -> double {
         if (!part) return A_io[(size_t)pair * NN * NN + x + y * NN];
@@ -418,11 +475,13 @@ k_solve_cross(const double *__restrict__ part, int nsplit, int full_part, double
         D[x] = entry(x, x);
         Sc[x] = 1.0;
         Rc[x] = 1.0;
+        if (!LA) Sd[LA ? 0 : x] = 1.0;
         if (dexp && rank == 0) dexp[(size_t)pair * NN + x] = D[x] > 0.0 ? (ilogb(D[x]) >> 1) : 0;
     }
     if (tid == 0) {
         s_own = h;
-        s_renorm = 0;
+        s_bad[0] = s_bad[1] = 0;
+        for (int w = 0; w < R::kHelpers; ++w) s_renorm[0][w] = s_renorm[1][w] = 0;
     }
     for (int e = tid; e < P * NN; e += kT) {
         const int kl = e / NN, y = e % NN;
@@ -500,49 +559,38 @@ k_solve_cross(const double *__restrict__ part, int nsplit, int full_part, double
         }
     }
     __syncthreads();
-    // (t, c) of the owned pairs for step s into every CTA (buffer s & 1)
-    auto put_params = [&](int s, int k, double t, double c, double qv, double apq, int fl) {
-        const int b = s & 1;
-        for (int r = 0; r < C; ++r) {
-            *cluster.map_shared_rank(&T[b][k], r) = t;
-            *cluster.map_shared_rank(&Cc[b][k], r) = c;
-            *cluster.map_shared_rank(&Qv[b][k], r) = qv;
-            *cluster.map_shared_rank(&Apq[b][k], r) = apq;
-            *cluster.map_shared_rank(&Fl[b][k], r) = fl;
+    const int warp = tid >> 5, lane = tid & 31;
+    // Lanes l, l + P, ... of a warp form the same rotation, that of owned pair
+    // l < P, and each writes it into every (32 / P)-th CTA.
+    constexpr int kRep = 32 / P;
+    const int ll = lane % P, rep = lane / P;
+    auto publish = [&](int s, double t, double al, double be, double c, double apq, int fl) {
+        const int bn = s & 1, k = k0 + ll;
+        for (int r = rep; r < C; r += kRep) {
+            cluster.map_shared_rank(&rt, r)->put(bn, k, t, al, be, c, apq, fl);
+            if (fl & kPairRank) *cluster.map_shared_rank(&s_bad[bn], r) = 1;
         }
     };
-    auto params_out = [&](int s) {
-        if (tid < P) {
-            const int kl = tid, k = k0 + kl, p = k, q = h + (k + s) % h;
-            const double apq = (Sc[p] * Sc[q]) * fix[kl * NN + q];  // true a_pq
-            const double app = D[p], aqq = D[q];
-            const int hyp = (sg[p] == sg[q]) ? -1 : 1;
-            double t, c, qv;
-            const int fl = pair_decision_fast(app, aqq, apq, hyp, tol, t, c, qv);
-            put_params(s, k, t, c, qv, apq, fl);
-        }
-    };
-    if (s0 < h) params_out(s0);
+    if (s0 < h && warp == 0) {  // the first step's rotations: scales 1
+        const int k = k0 + ll, q = h + (k + s0) % h, hyp = (sg[k] == sg[q]) ? -1 : 1;
+        double t, c = 1.0;
+        const double apq = (Sc[k] * Sc[q]) * fix[ll * NN + q];  // true a_pq
+        const int fl = pair_tangent(D[k], D[q], apq, hyp, tol, t);
+        if (LA && (fl & kPairRot)) c = rotation_cosine(t, hyp, pair_how(fl));
+        publish(s0, t, hyp < 0 ? -t : t, t, c, apq, fl);
+    }
     cluster.sync();
 
-    // Warp 0 works one step ahead: at the top of step s lane kl < P reads the
-    // four entries of its rows (k, q_k) in the columns (j, q') of pair
-    // j = k + 1 and the diagonal values a_kk, a_q'q', forms the step-s values
-    // of a_kq' and of the two diagonal entries with the same operations as the
-    // bulk update below, and computes the (t, c) of pair (k, q') for step
-    // s + 1 while warps 1..8 update the rows (named barrier 1).
-    // Without the look-ahead (LA = false) every warp mixes and the owners
-    // compute the next parameters after the update.
-    constexpr int kMixThreads = LA ? kT - 32 : kT;
-    const int warp = tid >> 5, lane = tid & 31;
     int total = 0, bad = 0, s_end = h - 1;
-    int big = 0;  // a rotation of pair tid had |t| > tstop (Eq. 4.2 code (11)_2)
-    const int mt = LA ? tid - 32 : tid;  // mixing thread index (warps 1.. with the look-ahead)
+    int big = 0;  // a rotation of the lane's pair had |t| > tstop (Eq. 4.2 code (11)_2)
+    const int mt = 32 * R::mixer(warp) + lane;  // mixing thread index (mixing warps)
     for (int s = s0; s < h; ++s) {
         const int b = s & 1;
         auto slot = [&](int kl) { return (kl + s) % (P + 1); };
         // scales out of range after the last step: the block back to s = r = 1
-        if (s_renorm) {
+        int renorm = s_renorm[b][0];
+        if (R::kHelpers > 1) renorm |= s_renorm[b][R::kHelpers - 1];
+        if (renorm) {
             for (int e = tid; e < (2 * P + RW) * NN; e += kT) {
                 const int r = e / NN, y = e % NN;
                 if (r < 2 * P) {
@@ -554,53 +602,38 @@ k_solve_cross(const double *__restrict__ part, int nsplit, int full_part, double
                 }
             }
             __syncthreads();
-            for (int x = tid; x < NN; x += kT) Sc[x] = Rc[x] = 1.0;
-            if (tid == 0) s_renorm = 0;
+            for (int x = tid; x < NN; x += kT) {
+                Sc[x] = Rc[x] = 1.0;
+                if (!LA) Sd[LA ? 0 : x] = 1.0;
+            }
             __syncthreads();
         }
-        double nx_t = 0.0, nx_c = 1.0, nx_qv = 1.0, nx_apq = 0.0;
-        int nx_fl = 0;
-        double e_kj = 0.0, e_kq = 0.0, e_qj = 0.0, e_qq = 0.0, d_k = 0.0, d_q = 0.0, s_k = 1.0, s_q = 1.0;
-        const bool ahead = LA && warp == 0 && lane < P && s + 1 < h;
-        if (ahead) {
-            const int kl = lane, k = k0 + kl, j = (k + 1) % h, q2 = h + (j + s) % h;
-            const double *rk = fix + kl * NN, *rq = mov + ((kl + s) % (P + 1)) * NN;
-            e_kj = rk[j];
-            e_kq = rk[q2];
-            e_qj = rq[j];
-            e_qq = rq[q2];
-            d_k = D[k];
-            d_q = D[q2];
-            s_k = Sc[k];
-            s_q = Sc[q2];
-        }
-        // the step's coefficients from its starting scales (alpha by threads
-        // [0, h), beta by [h, 2h): two FP64 instructions per warp)
-        if (mt >= 0 && mt < 2 * h && (Fl[b][mt % h] & 1)) {
-            const int j = mt % h, p = j, q = h + (j + s) % h;
-            const double t = T[b][j];
-            if (mt < h) Al[j] = ((sg[p] == sg[q]) ? -t : t) * (Sc[q] * Rc[p]);
-            else Be[j] = t * (Sc[p] * Rc[q]);
-        }
-        // every CTA sees every pair's flags: the same decision everywhere
-        const int f = tid < h ? Fl[b][tid] : 0;
-        if (tbig && (f & 1) && fabs(T[b][tid]) > tstop) big = 1;
-        bad = __syncthreads_or(f & 2);
+        bad = s_bad[b];  // every CTA has the same word: the same decision everywhere
         if (bad) {
             s_end = s;
             break;
         }
-        // the step's rotations, counted by the warps holding the flags (one
-        // CTA barrier per step instead of two); lane 0 of warp w keeps warp
-        // w's count
-        if (warp * 32 < h) total += __popc(__ballot_sync(0xffffffffu, f & 1));
         if (LA && warp == 0) {
-            if (ahead) {
-                const int kl = lane, k = k0 + kl, j = (k + 1) % h, q2 = h + (j + s) % h, qk = h + (k + s) % h;
-                const int fk = Fl[b][k] & 1, fj = Fl[b][j] & 1;
-                const double tk = T[b][k], htk = (sg[k] == sg[qk]) ? -tk : tk;
-                const double tj = T[b][j];
-                const double alk = fk ? Al[k] : 0.0, bej = fj ? Be[j] : 0.0;
+            // One step ahead: lane ll reads the four entries of its rows (k, q_k)
+            // in the columns (j, q') of pair j = k + 1 and the diagonal values
+            // a_kk, a_q'q' and scales before the others change them (barrier
+            // kBarRead), forms the step-s values of a_kq' and of the two diagonal
+            // entries with the same operations as the bulk update, and the
+            // rotation of pair (k, q') for step s + 1.
+            const int kl = ll, k = k0 + kl, j = (k + 1) % h, q2 = h + (j + s) % h, qk = h + (k + s) % h;
+            const double *rk = fix + kl * NN, *rq = mov + slot(kl) * NN;
+            const double e_kj = rk[j], e_kq = rk[q2], e_qj = rq[j], e_qq = rq[q2];
+            const double d_k = D[k], d_q = D[q2], s_k = Sc[k], s_q = Sc[q2];
+            bar_arrive(kBarRead, kT);
+            double t = 0.0, c = 1.0, apq = 0.0;
+            int fl = 0;
+            const int hyp = (sg[k] == sg[q2]) ? -1 : 1;
+            if (s + 1 < h) {
+                const int fk = rt.flags(b, k) & kPairRot, fj = rt.flags(b, j) & kPairRot;
+                const double2 ta_k = rt.ta[b][k], bp_j = rt.bp[b][j];
+                const double tk = ta_k.x, htk = (sg[k] == sg[qk]) ? -tk : tk;
+                const double tj = rt.ta[b][j].x;
+                const double alk = ta_k.y, bej = bp_j.x;
                 double v;
                 if ((s & 1) == 0) {  // column mix (pair j), then row mix (pair k)
                     double r1 = e_kq, r2 = e_qq;
@@ -617,55 +650,180 @@ k_solve_cross(const double *__restrict__ part, int nsplit, int full_part, double
                     }
                     v = fj ? fma(bej, u1, u2) : u2;
                 }
-                const double app = fk ? fma(htk, Apq[b][k], d_k) : d_k;
-                const double aqq = fj ? fma(tj, Apq[b][j], d_q) : d_q;
-                // the step's new scales of rows k and q2 (as the update phase forms them)
-                const double sk = fk ? s_k * Cc[b][k] : s_k, sq = fj ? s_q * Cc[b][j] : s_q;
-                const double apq = (sk * sq) * v;
-                const int hyp = (sg[k] == sg[q2]) ? -1 : 1;
-                nx_fl = pair_decision_fast(app, aqq, apq, hyp, tol, nx_t, nx_c, nx_qv);
-                nx_apq = apq;
+                const double app = fk ? fma(htk, rt.bp[b][k].y, d_k) : d_k;
+                const double aqq = fj ? fma(tj, bp_j.y, d_q) : d_q;
+                // the step's new scales of rows k and q2 (as the helpers form them)
+                const double sk = fk ? s_k * rt.cf[b][LA ? k : 0].x : s_k, sq = fj ? s_q * rt.cf[b][LA ? j : 0].x : s_q;
+                apq = (sk * sq) * v;
+                fl = pair_tangent(app, aqq, apq, hyp, tol, t);
+                if (fl & kPairRot) c = rotation_cosine(t, hyp, pair_how(fl));
             }
-        } else {
+            __syncwarp();
+            if (s + 1 < h) {
+                bar_sync(kBarRatio, 32 * (1 + R::kHelpers));
+                publish(s + 1, t, (hyp < 0 ? -t : t) * Ra[k], t * Rb[k], c, apq, fl);
+            }
+        } else if (LA && warp >= 9) {
+            const int hw = warp - 9, j = 32 * hw + lane;
+            bar_sync(kBarRead, kT);
+            const int f = rt.flags(b, j);
+            bool out = false;
+            if (f & kPairRot) {
+                const int p = j, q = h + (j + s) % h;
+                const double t = rt.ta[b][j].x, apq = rt.bp[b][j].y;
+                const int hyp = (sg[p] == sg[q]) ? -1 : 1;
+                D[p] = fma(hyp < 0 ? -t : t, apq, D[p]);
+                D[q] = fma(t, apq, D[q]);
+                const double c = rt.cf[b][LA ? j : 0].x, np = Sc[p] * c, nq = Sc[q] * c;
+                Sc[p] = np;
+                Sc[q] = nq;
+                const double qv = rotation_reciprocal(t, hyp, pair_how(f), c);
+                Rc[p] = Rc[p] * qv;
+                Rc[q] = Rc[q] * qv;
+                out = scale_out_of_range(np) || scale_out_of_range(nq);
+                if (tbig && fabs(t) > tstop) big = 1;
+            }
+            total += __popc(__ballot_sync(0xffffffffu, f & kPairRot));
+            out = __any_sync(0xffffffffu, out);
+            if (lane == 0) s_renorm[b ^ 1][hw] = out;
+            bar_sync(kBarHelp, 32 * R::kHelpers);
+            // the ratios of the next step's coefficients (1 after a return to s = r = 1)
+            if (s + 1 < h) {
+                out = s_renorm[b ^ 1][0] | s_renorm[b ^ 1][R::kHelpers - 1];
+                const int p = j, q = h + (j + s + 1) % h;
+                Ra[j] = out ? 1.0 : Sc[q] * Rc[p];
+                Rb[j] = out ? 1.0 : Sc[p] * Rc[q];
+                bar_arrive(kBarRatio, 32 * (1 + R::kHelpers));
+            }
+        } else if (!LA && warp == 0) {
+            // the cosines and scales of the step, then the next rotations
+            const int j = lane;
+            const int f = j < h ? rt.flags(b, j) : 0;
+            bool out = false;
+            if (f & kPairRot) {
+                const int p = j, q = h + (j + s) % h;
+                const double t = rt.ta[b][j].x;
+                const int hyp = (sg[p] == sg[q]) ? -1 : 1;
+                const double c = rotation_cosine(t, hyp, pair_how(f)), np = Sc[p] * c, nq = Sc[q] * c;
+                Sc[p] = np;
+                Sc[q] = nq;
+                out = scale_out_of_range(np) || scale_out_of_range(nq);
+            }
+            out = __any_sync(0xffffffffu, out);
+            if (lane == 0) s_renorm[b ^ 1][0] = out;
+            __syncwarp();
+            const int xp = k0 + ll, xq = h + (xp + s + 1) % h;
+            const int hyp = (sg[xp] == sg[xq]) ? -1 : 1;
+            const double ss = Sc[xp] * Sc[xq];
+            bar_sync(kBarDone, 64 + kMixThreads);
+            if (s + 1 < h) {
+                const double app = D[xp], aqq = D[xq], apq = ss * fix[ll * NN + xq];  // true a_pq
+                const RotStart rs = rotation_start(app, aqq, apq, hyp);
+                bar_sync(kBarTest, 64);
+                double t = 0.0;
+                int fl = 0;
+                if (!pass[LA ? 0 : lane]) {
+                    const int how = rotation_tangent(rs, app, aqq, apq, hyp, t);
+                    fl = pair_flags(how);
+                    if (!how) t = 0.0;
+                }
+                __syncwarp();
+                bar_sync(kBarRatio, 64);
+                publish(s + 1, t, (hyp < 0 ? -t : t) * Ra[xp], t * Rb[xp], 1.0, apq, fl);
+            }
+        } else if (!LA && warp == 4) {
+            // the diagonal and the counts, then the next pairs' tests
+            const int j = lane;
+            const int f = j < h ? rt.flags(b, j) : 0;
+            if (f & kPairRot) {
+                const int p = j, q = h + (j + s) % h;
+                const double t = rt.ta[b][j].x, apq = rt.bp[b][j].y;
+                D[p] = fma(sg[p] == sg[q] ? -t : t, apq, D[p]);
+                D[q] = fma(t, apq, D[q]);
+                if (tbig && fabs(t) > tstop) big = 1;
+            }
+            total += __popc(__ballot_sync(0xffffffffu, f & kPairRot));
+            const int xp = k0 + ll, xq = h + (xp + s + 1) % h;
+            bar_sync(kBarDone, 64 + kMixThreads);
+            if (s + 1 < h) {
+                pass[LA ? 0 : lane] = pair_passes(D[xp], D[xq], (Sc[xp] * Sc[xq]) * fix[ll * NN + xq], tol);
+                bar_arrive(kBarTest, 64);
+            }
+        } else if (!LA && warp == 11) {
+            // the reciprocals, and the ratios of the next step's coefficients
+            // (1 after a return to s = r = 1)
+            const int j = lane;
+            const int f = j < h ? rt.flags(b, j) : 0;
+            bool out = false;
+            if (f & kPairRot) {
+                const int p = j, q = h + (j + s) % h;
+                const double t = rt.ta[b][j].x;
+                const int hyp = (sg[p] == sg[q]) ? -1 : 1;
+                const double c = rotation_cosine(t, hyp, pair_how(f));
+                const double np = Sd[LA ? 0 : p] * c, nq = Sd[LA ? 0 : q] * c;
+                Sd[LA ? 0 : p] = np;
+                Sd[LA ? 0 : q] = nq;
+                const double qv = rotation_reciprocal(t, hyp, pair_how(f), c);
+                Rc[p] = Rc[p] * qv;
+                Rc[q] = Rc[q] * qv;
+                out = scale_out_of_range(np) || scale_out_of_range(nq);
+            }
+            out = __any_sync(0xffffffffu, out);
+            __syncwarp();
+            if (s + 1 < h) {
+                if (j < h) {
+                    const int p = j, q = h + (j + s + 1) % h;
+                    Ra[j] = out ? 1.0 : Sd[LA ? 0 : q] * Rc[p];
+                    Rb[j] = out ? 1.0 : Sd[LA ? 0 : p] * Rc[q];
+                }
+                __syncwarp();
+                bar_arrive(kBarRatio, 64);
+            }
+        } else if (R::mixes(warp)) {
+            if (LA) bar_sync(kBarRead, kT);
             // The column mix on every owned row of A (and of W): pair j's columns
             // j and h + (j + s) mod h.  A thread keeps one pair (its rotation in
             // registers) and walks rows; consecutive threads take consecutive
-            // pairs, so a warp's loads of one row are consecutive words.
-            auto col_mix = [&](bool with_w) {
+            // pairs, so a warp's loads of one row are consecutive words.  The
+            // second of the two mixes leaves zeros at an owned pair's own entries.
+            auto col_mix = [&](bool with_w, bool last) {
                 static_assert(kMixThreads % h == 0, "whole rows per pass");
                 const int j = mt % h;
-                if (!(Fl[b][j] & 1)) return;
+                if (!(rt.flags(b, j) & kPairRot)) return;
                 const int p = j, q = h + (j + s) % h;
-                const double al = Al[j], be = Be[j];
+                const double al = rt.ta[b][j].y, be = rt.bp[b][j].x;
                 const int nrows = 2 * P + (with_w ? RW : 0);
                 for (int r = mt / h; r < nrows; r += kMixThreads / h) {
                     double *row = r < P ? fix + r * NN : (r < 2 * P ? mov + slot(r - P) * NN : Wl + (r - 2 * P) * NN);
                     const double a = row[p], bb = row[q];
-                    row[p] = fma(al, bb, a);
-                    row[q] = fma(be, a, bb);
+                    const bool own = last && (r < P ? r : r - P) == j - k0;
+                    row[p] = own ? 0.0 : fma(al, bb, a);
+                    row[q] = own ? 0.0 : fma(be, a, bb);
                 }
             };
             // The row mix of every owned pair: rows k and its partner, every
             // column; a thread keeps one pair and walks columns.  With W, also
             // W's column mix (as in col_mix, on W's rows only).
-            auto row_mix = [&](bool with_w) {
+            auto row_mix = [&](bool with_w, bool last) {
                 static_assert(kMixThreads % P == 0, "threads split evenly over the owned pairs");
                 constexpr int TP = kMixThreads / P;  // threads per owned pair
                 const int kl = mt / TP, k = k0 + kl;
-                if (Fl[b][k] & 1) {
-                    const double al = Al[k], be = Be[k];
+                if (rt.flags(b, k) & kPairRot) {
+                    const double al = rt.ta[b][k].y, be = rt.bp[b][k].x;
+                    const int qk = h + (k + s) % h;
                     double *rp = fix + kl * NN, *rq = mov + slot(kl) * NN;
                     for (int y = mt % TP; y < NN; y += TP) {
                         const double a = rp[y], bb = rq[y];
-                        rp[y] = fma(al, bb, a);
-                        rq[y] = fma(be, a, bb);
+                        const bool own = last && (y == k || y == qk);
+                        rp[y] = own ? 0.0 : fma(al, bb, a);
+                        rq[y] = own ? 0.0 : fma(be, a, bb);
                     }
                 }
                 if (!with_w) return;
                 const int j = mt % h;
-                if (!(Fl[b][j] & 1)) return;
+                if (!(rt.flags(b, j) & kPairRot)) return;
                 const int pw = j, qw = h + (j + s) % h;
-                const double al = Al[j], be = Be[j];
+                const double al = rt.ta[b][j].y, be = rt.bp[b][j].x;
                 for (int x = mt / h; x < RW; x += kMixThreads / h) {
                     double *row = Wl + x * NN;
                     const double a = row[pw], bb = row[qw];
@@ -674,58 +832,26 @@ k_solve_cross(const double *__restrict__ part, int nsplit, int full_part, double
                 }
             };
             if ((s & 1) == 0) {
-                col_mix(true);
-                mix_sync<LA>(kMixThreads);
-                row_mix(false);
+                col_mix(true, false);
+                bar_sync(kBarMix, kMixThreads);
+                row_mix(false, true);
             } else {
-                row_mix(true);
-                mix_sync<LA>(kMixThreads);
-                col_mix(false);
+                row_mix(true, false);
+                bar_sync(kBarMix, kMixThreads);
+                col_mix(false, true);
             }
-            mix_sync<LA>(kMixThreads);
-            // Eq. 2.6 on the replicated diagonal and the owned pairs' own
-            // stored entries to 0 (threads [0, h)), the new scales (threads
-            // [h, 2h)) and their reciprocals (threads [2h, 3h)) of the rotated
-            // rows: three warp groups, so that no warp's chain of FP64
-            // instructions (one issues every 64 cycles) holds up the step
-            static_assert(kMixThreads >= 3 * h, "three groups of h mixing threads");
-            if (mt < 3 * h && (Fl[b][mt % h] & 1)) {
-                const int j = mt % h, p = j, q = h + (j + s) % h;
-                if (mt < h) {
-                    const double t = T[b][j], ht = (sg[p] == sg[q]) ? -t : t, apq = Apq[b][j];
-                    D[p] = fma(ht, apq, D[p]);
-                    D[q] = fma(t, apq, D[q]);
-                    if (p >= k0 && p < k0 + P) {
-                        const int kl = p - k0;
-                        double *rp = fix + kl * NN, *rq = mov + slot(kl) * NN;
-                        rp[p] = 0.0;
-                        rp[q] = 0.0;
-                        rq[q] = 0.0;
-                        rq[p] = 0.0;
-                    }
-                } else if (mt < 2 * h) {
-                    const double c = Cc[b][j];
-                    Sc[p] = Sc[p] * c;
-                    Sc[q] = Sc[q] * c;
-                    if (scale_out_of_range(Sc[p]) || scale_out_of_range(Sc[q])) s_renorm = 1;
-                } else {
-                    const double qv = Qv[b][j];
-                    Rc[p] = Rc[p] * qv;
-                    Rc[q] = Rc[q] * qv;
-                }
+            if (LA) bar_sync(kBarMix, kMixThreads);
+            else bar_sync(kBarDone, 64 + kMixThreads);
+            if (s + 1 < h) {
+                // hand the first pair's partner row to the previous CTA (its last
+                // pair's row at step s + 1, in the slot that is free during step s)
+                const int dst = (rank + C - 1) % C;
+                const double *src = mov + slot(0) * NN;
+                double *rdst = cluster.map_shared_rank(mov, dst) + ((P + s) % (P + 1)) * NN;
+                for (int y = mt; y < NN; y += kMixThreads) rdst[y] = src[y];
             }
         }
-        __syncthreads();
-        if (s + 1 < h) {
-            // hand the first pair's partner row to the previous CTA (its last
-            // pair's row at step s + 1, in the slot that is free during step s)
-            const int dst = (rank + C - 1) % C;
-            double *src = mov + slot(0) * NN;
-            double *rdst = cluster.map_shared_rank(mov, dst) + ((P + s) % (P + 1)) * NN;
-            for (int y = tid; y < NN; y += kT) rdst[y] = src[y];
-            if (!LA) params_out(s + 1);
-            if (ahead) put_params(s + 1, k0 + lane, nx_t, nx_c, nx_qv, nx_apq, nx_fl);
-        }
+        __syncwarp();
         cluster.sync();
     }
     // outputs: own rows of W (column-major W_P), and A_P when asked for
@@ -744,12 +870,12 @@ k_solve_cross(const double *__restrict__ part, int nsplit, int full_part, double
             ao[x + (size_t)y * NN] = x == y ? D[x] : (Sc[x] * Sc[y]) * mov[((kl + s_end) % (P + 1)) * NN + y];
         }
     }
-    if (lane == 0 && warp * 32 < h) s_tot[warp] = total;
+    if (lane == 0 && (LA ? warp >= 9 : warp == 4)) s_tot[LA ? warp - 9 : 0] = total;
     cluster.sync();
     const int any_big = tbig ? __syncthreads_or(big) : 0;
     if (rank == 0 && tid == 0) {
         total = 0;
-        for (int w = 0; w * 32 < h; ++w) total += s_tot[w];
+        for (int w = 0; w < R::kHelpers; ++w) total += s_tot[w];
         rotated[pair] = total;
         if (rot_count && total) atomicAdd(rot_count, (unsigned long long)total);
         if (bad && status) atomicExch(status, HSVD_ERR_RANK);
@@ -789,14 +915,15 @@ __device__ __forceinline__ int ring_buf_hi(int4 e) { return (e.z >> 8) & 0xff; }
 // (one free to receive); per step the row leaving its last slot is written
 // into the next CTA's free buffer, the only exchange of rows.  Both halves of
 // R^T A R are then local, as in the cross pass.  The entry a_lo,hi of a pair
-// is read from row lo (as the transposing kernel reads it), so the (t, c) of
+// is read from row lo (as the transposing kernel reads it), so the rotation of
 // a pair is formed by the CTA holding row lo at the end of the previous step:
 // the slot's own CTA, or the previous one when row lo is the row crossing
 // over.  The element operations and their order (column mix first on even
 // steps, row mix first on odd steps, Eq. 2.6 on the diagonal, zeros at the
-// pair) are those of k_solve_cluster in one-pass mode: the same bits.
+// pair) are those of k_solve_cluster in one-pass mode: the same bits.  The warps'
+// roles and what a rotation publishes are the cross pass's.
 template <int NN, int C, bool LA>
-__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(LA ? kCrossThreads : kClThreads, 3)
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(Role<LA>::kThreads, 2)
 k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double *__restrict__ A_io,
              const int8_t *__restrict__ sgn_cols, const int *__restrict__ col0,
              const int8_t *__restrict__ sgn_direct, double tol, const int4 *__restrict__ ring,
@@ -804,9 +931,10 @@ k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double 
              int *__restrict__ status, int *__restrict__ dexp, const int *__restrict__ visit,
              float *__restrict__ trace, double tstop, int *__restrict__ tbig) {
     constexpr int h = NN / 2, P = h / C, RW = NN / C, B = NN / 2, NBUF = 2 * P + 1;
-    constexpr int kT = LA ? kCrossThreads : kClThreads;
+    using R = Role<LA>;
+    constexpr int kT = R::kThreads;
     static_assert(P * C == h && RW * C == NN, "the slots and rows split evenly over the cluster");
-    static_assert(!LA || P + 1 <= 32, "the look-ahead warp has one lane per pair it forms");
+    static_assert(P + 1 <= 32 && h <= 32 * R::kHelpers, "one lane per pair formed, one helper lane per pair");
     static_assert(NBUF <= 255, "buffer indices fit the table's byte fields");
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
@@ -824,13 +952,14 @@ k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double 
     double *Wl = pool + NBUF * NN;   // [RW][NN] rows w0 .. w0 + RW - 1 of W_P
     __shared__ double D[NN];
     __shared__ int sg[NN];
-    __shared__ double T[2][h], Cc[2][h], Qv[2][h], Apq[2][h];  // Apq: the true a_pq
-    __shared__ int Fl[2][h];         // bit 0: rotate, bit 1: rank deficient
+    __shared__ __align__(16) Rots<h, LA> rt;
+    __shared__ double Ra[h], Rb[h];    // the next step's scale ratios
+    __shared__ double Sd[LA ? 1 : NN];  // the scales again, the ratio warp's own
+    __shared__ int pass[LA ? 1 : 32];   // the next step's pairs that pass Eq. 2.3
     __shared__ double Sc[NN], Rc[NN];  // column scales of the stored block and their reciprocals
-    __shared__ double Al[h], Be[h];    // the step's scaled-rotation coefficients
-    __shared__ int s_tot[2];           // rotations counted by warps 0 and 1
-    static_assert(h <= 64, "the rotation count lives in warps 0 and 1");
-    __shared__ int s_renorm;
+    __shared__ int s_renorm[2][R::kHelpers];  // scales out of range before the step (by parity)
+    __shared__ int s_bad[2];                  // a rank-deficient pair in the step (by parity)
+    __shared__ int s_tot[R::kHelpers];        // rotations counted by the helpers
     __shared__ int4 tb[3][h];        // ring table rows of steps s, s + 1, s + 2 (at step % 3)
     __shared__ double tr_max[C], tr_sum[C], tr_red[2][kT / 32];
 
@@ -849,9 +978,13 @@ k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double 
         D[x] = entry(x, x);
         Sc[x] = 1.0;
         Rc[x] = 1.0;
+        if (!LA) Sd[LA ? 0 : x] = 1.0;
         if (dexp && rank == 0) dexp[(size_t)pair * NN + x] = D[x] > 0.0 ? (ilogb(D[x]) >> 1) : 0;
     }
-    if (tid == 0) s_renorm = 0;
+    if (tid == 0) {
+        s_bad[0] = s_bad[1] = 0;
+        for (int w = 0; w < R::kHelpers; ++w) s_renorm[0][w] = s_renorm[1][w] = 0;
+    }
     for (int e = tid; e < 2 * h; e += kT) tb[e / h][e % h] = ring[e];
     __syncthreads();
     // rows of the owned slots at step 0, W = I
@@ -914,17 +1047,7 @@ k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double 
         *cluster.map_shared_rank(&tr_max[rank], 0) = rec_max;
         *cluster.map_shared_rank(&tr_sum[rank], 0) = rec_sum;
     }
-    // (t, c) of a pair into every CTA (buffer s & 1)
-    auto put_params = [&](int s, int k, double t, double c, double qv, double apq, int fl) {
-        const int b = s & 1;
-        for (int r = 0; r < C; ++r) {
-            *cluster.map_shared_rank(&T[b][k], r) = t;
-            *cluster.map_shared_rank(&Cc[b][k], r) = c;
-            *cluster.map_shared_rank(&Qv[b][k], r) = qv;
-            *cluster.map_shared_rank(&Apq[b][k], r) = apq;
-            *cluster.map_shared_rank(&Fl[b][k], r) = fl;
-        }
-    };
+    const int warp = tid >> 5, lane = tid & 31;
     // Lane l <= P forms the step-s pair of slot k0 + l (l = P: the next CTA's
     // first slot) when this CTA holds its row lo at the end of step s - 1:
     // row lo stays in slot k0 + l, or arrives from slot k0 + l - 1 (local for
@@ -934,34 +1057,42 @@ k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double 
         const bool lo_arr = e.w & 1;
         return l < P ? !(lo_arr && l == 0) : lo_arr;
     };
-    // step 0: every CTA forms the pairs of its own slots
-    if (tid < P) {
-        const int k = k0 + tid;
-        const int4 e = tb[0][k];
-        const double apq = (Sc[e.x] * Sc[e.y]) * pool[ring_buf_lo(e) * NN + e.y];
-        const int hyp = (sg[e.x] == sg[e.y]) ? -1 : 1;
-        double t, c, qv;
-        const int fl = pair_decision_fast(D[e.x], D[e.y], apq, hyp, tol, t, c, qv);
-        put_params(0, k, t, c, qv, apq, fl);
+    // Lanes l, l + (P + 1), ... of a warp form the same rotation, l <= P, and each
+    // writes it into every kRep-th CTA.
+    constexpr int kRep = 32 / (P + 1);
+    const int ll = lane % (P + 1), rep = lane / (P + 1);
+    auto publish = [&](int s, bool mine, double t, double al, double be, double c, double apq, int fl) {
+        if (!mine || rep >= kRep) return;
+        const int bn = s & 1, k = (k0 + ll) % h;
+        for (int r = rep; r < C; r += kRep) {
+            cluster.map_shared_rank(&rt, r)->put(bn, k, t, al, be, c, apq, fl);
+            if (fl & kPairRank) *cluster.map_shared_rank(&s_bad[bn], r) = 1;
+        }
+    };
+    if (warp == 0) {  // step 0 (scales 1): every CTA forms the pairs of its own slots
+        double t = 0.0, c = 1.0, apq = 0.0;
+        int fl = 0, hyp = 1;
+        if (ll < P) {
+            const int4 e = tb[0][k0 + ll];
+            apq = (Sc[e.x] * Sc[e.y]) * pool[ring_buf_lo(e) * NN + e.y];
+            hyp = (sg[e.x] == sg[e.y]) ? -1 : 1;
+            fl = pair_tangent(D[e.x], D[e.y], apq, hyp, tol, t);
+            if (LA && (fl & kPairRot)) c = rotation_cosine(t, hyp, pair_how(fl));
+        }
+        publish(0, ll < P, t, hyp < 0 ? -t : t, t, c, apq, fl);
     }
     cluster.sync();
 
-    // Warp 0 works one step ahead (LA): lane l reads, at the top of step s,
-    // the four entries of the rows of pair i (the slot holding row lo of the
-    // step-(s+1) pair) in the columns of pair j (the slot holding its row hi)
-    // and the two diagonal values, forms their step-s values with the
-    // operations of the bulk update and the (t, c) of the step-(s+1) pair,
-    // while warps 1.. update the rows (named barrier 1).
-    constexpr int kMixThreads = LA ? kT - 32 : kT;
-    const int warp = tid >> 5, lane = tid & 31;
     int total = 0, bad = 0, s_end = NN - 1;
-    int big = 0;  // a rotation of pair tid had |t| > tstop (Eq. 4.2 code (11)_2)
-    const int mt = LA ? tid - 32 : tid;  // mixing thread index (warps 1.. with the look-ahead)
+    int big = 0;  // a rotation of the lane's pair had |t| > tstop (Eq. 4.2 code (11)_2)
+    const int mt = 32 * R::mixer(warp) + lane;  // mixing thread index (mixing warps)
     for (int s = 0; s < NN; ++s) {
         const int b = s & 1;
-        const int4 *cur = tb[s % 3];
+        const int4 *cur = tb[s % 3], *nxt = tb[(s + 1) % 3];
         // scales out of range after the last step: the block back to s = r = 1
-        if (s_renorm) {
+        int renorm = s_renorm[b][0];
+        if (R::kHelpers > 1) renorm |= s_renorm[b][R::kHelpers - 1];
+        if (renorm) {
             for (int e = tid; e < (2 * P + RW) * NN; e += kT) {
                 const int r = e / NN, y = e % NN;
                 if (r < 2 * P) {
@@ -973,65 +1104,52 @@ k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double 
                 }
             }
             __syncthreads();
-            for (int x = tid; x < NN; x += kT) Sc[x] = Rc[x] = 1.0;
-            if (tid == 0) s_renorm = 0;
+            for (int x = tid; x < NN; x += kT) {
+                Sc[x] = Rc[x] = 1.0;
+                if (!LA) Sd[LA ? 0 : x] = 1.0;
+            }
             __syncthreads();
         }
-        double nx_t = 0.0, nx_c = 1.0, nx_qv = 1.0, nx_apq = 0.0;
-        int nx_fl = 0;
-        double e_pp = 0.0, e_pq = 0.0, e_qp = 0.0, e_qq = 0.0, d_lo = 0.0, d_hi = 0.0, s_lo = 1.0, s_hi = 1.0;
-        int si = 0, sj = 0;
-        bool lo_p = false, hi_p = false, trig_i = false, trig_j = false, trig_n = false;
-        const bool ahead = LA && warp == 0 && lane <= P && s + 1 < NN && forms(s + 1, lane);
-        if (ahead) {
-            const int k = (k0 + lane) % h;
-            const int4 ne = tb[(s + 1) % 3][k];
-            const bool lo_arr = ne.w & 1;
-            si = lo_arr ? (k + h - 1) % h : k;
-            sj = lo_arr ? k : (k + h - 1) % h;
-            const int4 fi = cur[si], fj = cur[sj];
-            const double *rp = pool + ring_buf_lo(fi) * NN, *rq = pool + ring_buf_hi(fi) * NN;
-            e_pp = rp[fj.x];
-            e_pq = rp[fj.y];
-            e_qp = rq[fj.x];
-            e_qq = rq[fj.y];
-            d_lo = D[ne.x];
-            d_hi = D[ne.y];
-            s_lo = Sc[ne.x];
-            s_hi = Sc[ne.y];
-            lo_p = ne.x == fi.x;  // row lo is pair i's first row
-            hi_p = ne.y == fj.x;  // column hi is pair j's first column
-            trig_i = sg[fi.x] == sg[fi.y];
-            trig_j = sg[fj.x] == sg[fj.y];
-            trig_n = sg[ne.x] == sg[ne.y];
-        }
-        // the step's coefficients from its starting scales (alpha by threads
-        // [0, h), beta by [h, 2h))
-        if (mt >= 0 && mt < 2 * h && (Fl[b][mt % h] & 1)) {
-            const int j = mt % h, p = cur[j].x, q = cur[j].y;
-            const double t = T[b][j];
-            if (mt < h) Al[j] = ((sg[p] == sg[q]) ? -t : t) * (Sc[q] * Rc[p]);
-            else Be[j] = t * (Sc[p] * Rc[q]);
-        }
-        // every CTA sees every pair's flags: the same decision everywhere
-        const int f = tid < h ? Fl[b][tid] : 0;
-        if (tbig && (f & 1) && fabs(T[b][tid]) > tstop) big = 1;
-        bad = __syncthreads_or(f & 2);
+        bad = s_bad[b];  // every CTA has the same word: the same decision everywhere
         if (bad) {
             s_end = s;
             break;
         }
-        // the step's rotations, counted by the warps holding the flags (one
-        // CTA barrier per step instead of two); lane 0 of warp w keeps warp
-        // w's count
-        if (warp * 32 < h) total += __popc(__ballot_sync(0xffffffffu, f & 1));
         if (LA && warp == 0) {
-            if (ahead) {
-                const int ri = Fl[b][si] & 1, rj = Fl[b][sj] & 1;
-                const double ti = T[b][si], hti = trig_i ? -ti : ti;
-                const double tj = T[b][sj], htj = trig_j ? -tj : tj;
-                const double ali = ri ? Al[si] : 0.0, bei = ri ? Be[si] : 0.0;
-                const double alj = rj ? Al[sj] : 0.0, bej = rj ? Be[sj] : 0.0;
+            // One step ahead: lane ll reads the four entries of the rows of pair i
+            // (the slot holding row lo of the step-(s+1) pair) in the columns of
+            // pair j (the slot holding its row hi) and the two diagonal values and
+            // scales before the others change them (barrier kBarRead), forms
+            // their step-s values with the operations of the bulk update and the
+            // rotation of the step-(s+1) pair.
+            const bool act = s + 1 < NN && forms(s + 1, ll);
+            const int k = (k0 + ll) % h;
+            const int4 ne = s + 1 < NN ? nxt[k] : cur[k];
+            const bool lo_arr = ne.w & 1;
+            const int si = lo_arr ? (k + h - 1) % h : k, sj = lo_arr ? k : (k + h - 1) % h;
+            const int4 fi = cur[si], fj = cur[sj];
+            double e_pp = 0.0, e_pq = 0.0, e_qp = 0.0, e_qq = 0.0;
+            if (act) {
+                const double *rp = pool + ring_buf_lo(fi) * NN, *rq = pool + ring_buf_hi(fi) * NN;
+                e_pp = rp[fj.x];
+                e_pq = rp[fj.y];
+                e_qp = rq[fj.x];
+                e_qq = rq[fj.y];
+            }
+            const double d_lo = D[ne.x], d_hi = D[ne.y], s_lo = Sc[ne.x], s_hi = Sc[ne.y];
+            bar_arrive(kBarRead, kT);
+            const bool lo_p = ne.x == fi.x;  // row lo is pair i's first row
+            const bool hi_p = ne.y == fj.x;  // column hi is pair j's first column
+            const bool trig_i = sg[fi.x] == sg[fi.y], trig_j = sg[fj.x] == sg[fj.y];
+            const int hyp = sg[ne.x] == sg[ne.y] ? -1 : 1;
+            double t = 0.0, c = 1.0, apq = 0.0;
+            int fl = 0;
+            if (act) {
+                const int ri = rt.flags(b, si) & kPairRot, rj = rt.flags(b, sj) & kPairRot;
+                const double2 ta_i = rt.ta[b][si], ta_j = rt.ta[b][sj], bp_i = rt.bp[b][si], bp_j = rt.bp[b][sj];
+                const double ti = ta_i.x, hti = trig_i ? -ti : ti;
+                const double tj = ta_j.x, htj = trig_j ? -tj : tj;
+                const double ali = ta_i.y, bei = bp_i.x, alj = ta_j.y, bej = bp_j.x;
                 double v;
                 if ((s & 1) == 0) {  // column mix (pair j) of rows p_i, q_i, then row mix (pair i)
                     double up = hi_p ? e_pp : e_pq, uq = hi_p ? e_qp : e_qq;
@@ -1051,57 +1169,194 @@ k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double 
                     if (rj) v = hi_p ? fma(alj, wq, wp) : fma(bej, wp, wq);
                 }
                 // Eq. 2.6 on the two diagonal entries, the step's new scales of the two rows
-                const double app = ri ? fma(lo_p ? hti : ti, Apq[b][si], d_lo) : d_lo;
-                const double aqq = rj ? fma(hi_p ? htj : tj, Apq[b][sj], d_hi) : d_hi;
-                const double sl = ri ? s_lo * Cc[b][si] : s_lo, sh = rj ? s_hi * Cc[b][sj] : s_hi;
-                const double apq = (sl * sh) * v;
-                nx_fl = pair_decision_fast(app, aqq, apq, trig_n ? -1 : 1, tol, nx_t, nx_c, nx_qv);
-                nx_apq = apq;
+                const double app = ri ? fma(lo_p ? hti : ti, bp_i.y, d_lo) : d_lo;
+                const double aqq = rj ? fma(hi_p ? htj : tj, bp_j.y, d_hi) : d_hi;
+                const double sl = ri ? s_lo * rt.cf[b][LA ? si : 0].x : s_lo, sh = rj ? s_hi * rt.cf[b][LA ? sj : 0].x : s_hi;
+                apq = (sl * sh) * v;
+                fl = pair_tangent(app, aqq, apq, hyp, tol, t);
+                if (fl & kPairRot) c = rotation_cosine(t, hyp, pair_how(fl));
             }
-        } else {
+            __syncwarp();
+            if (s + 1 < NN) {
+                bar_sync(kBarRatio, 32 * (1 + R::kHelpers));
+                publish(s + 1, act, t, (hyp < 0 ? -t : t) * Ra[k], t * Rb[k], c, apq, fl);
+            }
+        } else if (LA && warp >= 9) {
+            const int hw = warp - 9, j = 32 * hw + lane;
+            bar_sync(kBarRead, kT);
+            const int f = rt.flags(b, j);
+            bool out = false;
+            if (f & kPairRot) {
+                const int p = cur[j].x, q = cur[j].y;
+                const double t = rt.ta[b][j].x, apq = rt.bp[b][j].y;
+                const int hyp = (sg[p] == sg[q]) ? -1 : 1;
+                D[p] = fma(hyp < 0 ? -t : t, apq, D[p]);
+                D[q] = fma(t, apq, D[q]);
+                const double c = rt.cf[b][LA ? j : 0].x, np = Sc[p] * c, nq = Sc[q] * c;
+                Sc[p] = np;
+                Sc[q] = nq;
+                const double qv = rotation_reciprocal(t, hyp, pair_how(f), c);
+                Rc[p] = Rc[p] * qv;
+                Rc[q] = Rc[q] * qv;
+                out = scale_out_of_range(np) || scale_out_of_range(nq);
+                if (tbig && fabs(t) > tstop) big = 1;
+            }
+            total += __popc(__ballot_sync(0xffffffffu, f & kPairRot));
+            out = __any_sync(0xffffffffu, out);
+            if (lane == 0) s_renorm[b ^ 1][hw] = out;
+            bar_sync(kBarHelp, 32 * R::kHelpers);
+            // the ratios of the next step's coefficients (1 after a return to s = r = 1)
+            if (s + 1 < NN) {
+                out = s_renorm[b ^ 1][0] | s_renorm[b ^ 1][R::kHelpers - 1];
+                const int p = nxt[j].x, q = nxt[j].y;
+                Ra[j] = out ? 1.0 : Sc[q] * Rc[p];
+                Rb[j] = out ? 1.0 : Sc[p] * Rc[q];
+                bar_arrive(kBarRatio, 32 * (1 + R::kHelpers));
+            }
+        } else if (!LA && warp == 0) {
+            // the cosines and scales of the step, then the next rotations
+            const int j = lane;
+            const int f = j < h ? rt.flags(b, j) : 0;
+            bool out = false;
+            if (f & kPairRot) {
+                const int p = cur[j].x, q = cur[j].y;
+                const double t = rt.ta[b][j].x;
+                const int hyp = (sg[p] == sg[q]) ? -1 : 1;
+                const double c = rotation_cosine(t, hyp, pair_how(f)), np = Sc[p] * c, nq = Sc[q] * c;
+                Sc[p] = np;
+                Sc[q] = nq;
+                out = scale_out_of_range(np) || scale_out_of_range(nq);
+            }
+            out = __any_sync(0xffffffffu, out);
+            if (lane == 0) s_renorm[b ^ 1][0] = out;
+            __syncwarp();
+            const bool act = s + 1 < NN && forms(s + 1, ll);
+            const int k = (k0 + ll) % h;
+            const int4 e = s + 1 < NN ? nxt[k] : cur[k];
+            // row lo of the step-(s+1) pair, where it is at step s
+            const int4 at = cur[(e.w & 1) ? (k + h - 1) % h : k];
+            const double *row = pool + (at.x == e.x ? ring_buf_lo(at) : ring_buf_hi(at)) * NN;
+            const int xp = e.x, xq = e.y;
+            const int hyp = (sg[xp] == sg[xq]) ? -1 : 1;
+            const double ss = Sc[xp] * Sc[xq];
+            bar_sync(kBarDone, 64 + kMixThreads);
+            if (s + 1 < NN) {
+                const double app = D[xp], aqq = D[xq], apq = ss * row[xq];  // true a_pq
+                const RotStart rs = rotation_start(app, aqq, apq, hyp);
+                bar_sync(kBarTest, 64);
+                double t = 0.0;
+                int fl = 0;
+                if (!pass[LA ? 0 : lane]) {
+                    const int how = rotation_tangent(rs, app, aqq, apq, hyp, t);
+                    fl = pair_flags(how);
+                    if (!how) t = 0.0;
+                }
+                __syncwarp();
+                bar_sync(kBarRatio, 64);
+                publish(s + 1, act, t, (hyp < 0 ? -t : t) * Ra[k], t * Rb[k], 1.0, apq, fl);
+            }
+        } else if (!LA && warp == 4) {
+            // the diagonal and the counts, then the next pairs' tests
+            const int j = lane;
+            const int f = j < h ? rt.flags(b, j) : 0;
+            if (f & kPairRot) {
+                const int p = cur[j].x, q = cur[j].y;
+                const double t = rt.ta[b][j].x, apq = rt.bp[b][j].y;
+                D[p] = fma(sg[p] == sg[q] ? -t : t, apq, D[p]);
+                D[q] = fma(t, apq, D[q]);
+                if (tbig && fabs(t) > tstop) big = 1;
+            }
+            total += __popc(__ballot_sync(0xffffffffu, f & kPairRot));
+            const int k = (k0 + ll) % h;
+            const int4 e = s + 1 < NN ? nxt[k] : cur[k];
+            // row lo of the step-(s+1) pair, where it is at step s
+            const int4 at = cur[(e.w & 1) ? (k + h - 1) % h : k];
+            const double *row = pool + (at.x == e.x ? ring_buf_lo(at) : ring_buf_hi(at)) * NN;
+            const int xp = e.x, xq = e.y;
+            bar_sync(kBarDone, 64 + kMixThreads);
+            if (s + 1 < NN) {
+                pass[LA ? 0 : lane] = pair_passes(D[xp], D[xq], (Sc[xp] * Sc[xq]) * row[xq], tol);
+                bar_arrive(kBarTest, 64);
+            }
+        } else if (!LA && warp == 11) {
+            // the reciprocals, and the ratios of the next step's coefficients
+            // (1 after a return to s = r = 1)
+            const int j = lane;
+            const int f = j < h ? rt.flags(b, j) : 0;
+            bool out = false;
+            if (f & kPairRot) {
+                const int p = cur[j].x, q = cur[j].y;
+                const double t = rt.ta[b][j].x;
+                const int hyp = (sg[p] == sg[q]) ? -1 : 1;
+                const double c = rotation_cosine(t, hyp, pair_how(f));
+                const double np = Sd[LA ? 0 : p] * c, nq = Sd[LA ? 0 : q] * c;
+                Sd[LA ? 0 : p] = np;
+                Sd[LA ? 0 : q] = nq;
+                const double qv = rotation_reciprocal(t, hyp, pair_how(f), c);
+                Rc[p] = Rc[p] * qv;
+                Rc[q] = Rc[q] * qv;
+                out = scale_out_of_range(np) || scale_out_of_range(nq);
+            }
+            out = __any_sync(0xffffffffu, out);
+            __syncwarp();
+            if (s + 1 < NN) {
+                if (j < h) {
+                    const int p = nxt[j].x, q = nxt[j].y;
+                    Ra[j] = out ? 1.0 : Sd[LA ? 0 : q] * Rc[p];
+                    Rb[j] = out ? 1.0 : Sd[LA ? 0 : p] * Rc[q];
+                }
+                __syncwarp();
+                bar_arrive(kBarRatio, 64);
+            }
+        } else if (R::mixes(warp)) {
+            if (LA) bar_sync(kBarRead, kT);
             // the column mix on every held row of A (and of W): a thread keeps
-            // one pair (its rotation in registers) and walks rows
-            auto col_mix = [&](bool with_w) {
+            // one pair (its rotation in registers) and walks rows; the second of
+            // the two mixes leaves zeros at an owned pair's own entries
+            auto col_mix = [&](bool with_w, bool last) {
                 static_assert(kMixThreads % h == 0, "whole rows per pass");
                 const int j = mt % h;
-                if (!(Fl[b][j] & 1)) return;
+                if (!(rt.flags(b, j) & kPairRot)) return;
                 const int p = cur[j].x, q = cur[j].y;
-                const double al = Al[j], be = Be[j];
+                const double al = rt.ta[b][j].y, be = rt.bp[b][j].x;
                 const int nrows = 2 * P + (with_w ? RW : 0);
                 for (int r = mt / h; r < nrows; r += kMixThreads / h) {
                     double *row;
+                    bool own = false;
                     if (r < 2 * P) {
                         const int4 e = cur[k0 + (r >> 1)];
                         row = pool + ((r & 1) ? ring_buf_hi(e) : ring_buf_lo(e)) * NN;
+                        own = last && k0 + (r >> 1) == j;
                     } else {
                         row = Wl + (r - 2 * P) * NN;
                     }
                     const double a = row[p], bb = row[q];
-                    row[p] = fma(al, bb, a);
-                    row[q] = fma(be, a, bb);
+                    row[p] = own ? 0.0 : fma(al, bb, a);
+                    row[q] = own ? 0.0 : fma(be, a, bb);
                 }
             };
             // the row mix of every owned slot's pair, every column; with W,
             // also W's column mix
-            auto row_mix = [&](bool with_w) {
+            auto row_mix = [&](bool with_w, bool last) {
                 static_assert(kMixThreads % P == 0, "threads split evenly over the owned slots");
                 constexpr int TP = kMixThreads / P;  // threads per owned slot
                 const int kl = mt / TP, k = k0 + kl;
-                if (Fl[b][k] & 1) {
+                if (rt.flags(b, k) & kPairRot) {
                     const int4 e = cur[k];
-                    const double al = Al[k], be = Be[k];
+                    const double al = rt.ta[b][k].y, be = rt.bp[b][k].x;
                     double *rp = pool + ring_buf_lo(e) * NN, *rq = pool + ring_buf_hi(e) * NN;
                     for (int y = mt % TP; y < NN; y += TP) {
                         const double a = rp[y], bb = rq[y];
-                        rp[y] = fma(al, bb, a);
-                        rq[y] = fma(be, a, bb);
+                        const bool own = last && (y == e.x || y == e.y);
+                        rp[y] = own ? 0.0 : fma(al, bb, a);
+                        rq[y] = own ? 0.0 : fma(be, a, bb);
                     }
                 }
                 if (!with_w) return;
                 const int j = mt % h;
-                if (!(Fl[b][j] & 1)) return;
+                if (!(rt.flags(b, j) & kPairRot)) return;
                 const int pw = cur[j].x, qw = cur[j].y;
-                const double al = Al[j], be = Be[j];
+                const double al = rt.ta[b][j].y, be = rt.bp[b][j].x;
                 for (int x = mt / h; x < RW; x += kMixThreads / h) {
                     double *row = Wl + x * NN;
                     const double a = row[pw], bb = row[qw];
@@ -1110,52 +1365,19 @@ k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double 
                 }
             };
             if ((s & 1) == 0) {
-                col_mix(true);
-                mix_sync<LA>(kMixThreads);
-                row_mix(false);
+                col_mix(true, false);
+                bar_sync(kBarMix, kMixThreads);
+                row_mix(false, true);
             } else {
-                row_mix(true);
-                mix_sync<LA>(kMixThreads);
-                col_mix(false);
+                row_mix(true, false);
+                bar_sync(kBarMix, kMixThreads);
+                col_mix(false, true);
             }
-            mix_sync<LA>(kMixThreads);
-            // Eq. 2.6 on the replicated diagonal and the owned pairs' own
-            // stored entries to 0, the new scales and their reciprocals of
-            // the rotated rows, in three warp groups (as in the cross pass)
-            static_assert(kMixThreads >= 3 * h, "three groups of h mixing threads");
-            if (mt < 3 * h && (Fl[b][mt % h] & 1)) {
-                const int j = mt % h;
-                const int4 e = cur[j];
-                const int p = e.x, q = e.y;
-                if (mt < h) {
-                    const double t = T[b][j], ht = (sg[p] == sg[q]) ? -t : t, apq = Apq[b][j];
-                    D[p] = fma(ht, apq, D[p]);
-                    D[q] = fma(t, apq, D[q]);
-                    if (j >= k0 && j < k0 + P) {
-                        double *rp = pool + ring_buf_lo(e) * NN, *rq = pool + ring_buf_hi(e) * NN;
-                        rp[p] = 0.0;
-                        rp[q] = 0.0;
-                        rq[q] = 0.0;
-                        rq[p] = 0.0;
-                    }
-                } else if (mt < 2 * h) {
-                    const double c = Cc[b][j];
-                    Sc[p] = Sc[p] * c;
-                    Sc[q] = Sc[q] * c;
-                    if (scale_out_of_range(Sc[p]) || scale_out_of_range(Sc[q])) s_renorm = 1;
-                } else {
-                    const double qv = Qv[b][j];
-                    Rc[p] = Rc[p] * qv;
-                    Rc[q] = Rc[q] * qv;
-                }
-            }
-        }
-        __syncthreads();
-        if (s + 1 < NN) {
-            const int4 *nxt = tb[(s + 1) % 3];
-            // the row leaving the last owned slot: the row arriving in slot
-            // k0 + P at step s + 1, into its buffer in the next CTA
-            {
+            if (LA) bar_sync(kBarMix, kMixThreads);
+            else bar_sync(kBarDone, 64 + kMixThreads);
+            if (s + 1 < NN) {
+                // the row leaving the last owned slot: the row arriving in slot
+                // k0 + P at step s + 1, into its buffer in the next CTA
                 const int4 en = nxt[(k0 + P) % h];
                 const bool lo_arr = en.w & 1;
                 const int mv = lo_arr ? en.x : en.y, dbf = lo_arr ? ring_buf_lo(en) : ring_buf_hi(en);
@@ -1163,25 +1385,13 @@ k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double 
                 const int sbf = el.x == mv ? ring_buf_lo(el) : ring_buf_hi(el);
                 double *rdst = cluster.map_shared_rank(pool, (rank + 1) % C) + dbf * NN;
                 const double *src = pool + sbf * NN;
-                for (int y = tid; y < NN; y += kT) rdst[y] = src[y];
+                for (int y = mt; y < NN; y += kMixThreads) rdst[y] = src[y];
+                // the table row of step s + 2 into the slot of step s - 1
+                if (s + 2 < NN)
+                    for (int e = mt; e < h; e += kMixThreads) tb[(s + 2) % 3][e] = ring[(size_t)(s + 2) * h + e];
             }
-            if (!LA && tid <= P && forms(s + 1, tid)) {
-                // row lo of the step-(s+1) pair, where it is at step s
-                const int k = (k0 + tid) % h;
-                const int4 e = nxt[k];
-                const int4 fl = cur[(e.w & 1) ? (k + h - 1) % h : k];
-                const int bf = fl.x == e.x ? ring_buf_lo(fl) : ring_buf_hi(fl);
-                const double apq = (Sc[e.x] * Sc[e.y]) * pool[bf * NN + e.y];
-                const int hyp = (sg[e.x] == sg[e.y]) ? -1 : 1;
-                double t, c, qv;
-                const int fd = pair_decision_fast(D[e.x], D[e.y], apq, hyp, tol, t, c, qv);
-                put_params(s + 1, k, t, c, qv, apq, fd);
-            }
-            if (ahead) put_params(s + 1, (k0 + lane) % h, nx_t, nx_c, nx_qv, nx_apq, nx_fl);
-            // the table row of step s + 2 into the slot of step s - 1
-            if (s + 2 < NN)
-                for (int e = tid; e < h; e += kT) tb[(s + 2) % 3][e] = ring[(size_t)(s + 2) * h + e];
         }
+        __syncwarp();
         cluster.sync();
     }
     // outputs: own rows of W (column-major W_P), and A_P when asked for
@@ -1202,12 +1412,12 @@ k_solve_ring(const double *__restrict__ part, int nsplit, int full_part, double 
             ao[x + (size_t)y * NN] = x == y ? D[x] : (Sc[x] * Sc[y]) * pool[bf * NN + y];
         }
     }
-    if (lane == 0 && warp * 32 < h) s_tot[warp] = total;
+    if (lane == 0 && (LA ? warp >= 9 : warp == 4)) s_tot[LA ? warp - 9 : 0] = total;
     cluster.sync();
     const int any_big = tbig ? __syncthreads_or(big) : 0;
     if (rank == 0 && tid == 0) {
         total = 0;
-        for (int w = 0; w * 32 < h; ++w) total += s_tot[w];
+        for (int w = 0; w < R::kHelpers; ++w) total += s_tot[w];
         rotated[pair] = total;
         if (rot_count && total) atomicAdd(rot_count, (unsigned long long)total);
         if (bad && status) atomicExch(status, HSVD_ERR_RANK);
@@ -1239,13 +1449,15 @@ cudaError_t solve_cluster_impl(int npairs, const double *part, int nsplit, int f
     if (mode == 1) {
         constexpr int CX = CrossClusterOf<NN>::C, P = NN / 2 / CX, RX = NN / CX;
         const size_t smem_x = (size_t)(P * NN + (P + 1) * NN + RX * NN) * sizeof(double);
-        // the look-ahead warp pays at b = 64 (measured), not at b <= 32
+        // the look-ahead warp pays at b = 64, where mixing is the longer path; at
+        // b <= 32 it shares the FP64 pipe with the mix it should run beside
+        // (one step ahead: 6,700 cycles a step at b = 16 with the owner's
+        // parameters, against 7,000 without and 4,500 with the roles above)
         constexpr bool LA = NN >= 128;
-        constexpr int threads = LA ? kCrossThreads : kClThreads;
         cudaError_t e = cudaFuncSetAttribute(k_solve_cross<NN, CX, LA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem_x);
         if (e != cudaSuccess) return e;
-        k_solve_cross<NN, CX, LA><<<npairs * CX, threads, smem_x, st>>>(part, nsplit, full_part, A, sgn_cols, col0,
+        k_solve_cross<NN, CX, LA><<<npairs * CX, Role<LA>::kThreads, smem_x, st>>>(part, nsplit, full_part, A, sgn_cols, col0,
                                                                      sgn_direct, tol, Wp, rotated, rot_count,
                                                                      status, dexp, visit, trace, tstop, tbig);
         return cudaGetLastError();
@@ -1254,12 +1466,11 @@ cudaError_t solve_cluster_impl(int npairs, const double *part, int nsplit, int f
         constexpr int CX = CrossClusterOf<NN>::C, P = NN / 2 / CX, RX = NN / CX;
         const size_t smem_r = (size_t)((2 * P + 1) * NN + RX * NN) * sizeof(double);
         constexpr bool LA = NN >= 128;
-        constexpr int threads = LA ? kCrossThreads : kClThreads;
         const int4 *ring = reinterpret_cast<const int4 *>(tab_full + (size_t)NN * (NN / 2) * 2);
         cudaError_t e = cudaFuncSetAttribute(k_solve_ring<NN, CX, LA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem_r);
         if (e != cudaSuccess) return e;
-        k_solve_ring<NN, CX, LA><<<npairs * CX, threads, smem_r, st>>>(part, nsplit, full_part, A, sgn_cols, col0,
+        k_solve_ring<NN, CX, LA><<<npairs * CX, Role<LA>::kThreads, smem_r, st>>>(part, nsplit, full_part, A, sgn_cols, col0,
                                                                     sgn_direct, tol, ring, Wp, rotated, rot_count,
                                                                     status, dexp, visit, trace, tstop, tbig);
         return cudaGetLastError();

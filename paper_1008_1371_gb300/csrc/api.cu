@@ -1117,9 +1117,8 @@ int hsvd_shorten_qr(const double *G, int64_t m, int64_t n, int64_t ldg, double *
         Ws ws(st);
         double *A = ws.get<double>((size_t)m * n);
         double *qws = ws.get<double>(qr_workspace_doubles(n));
-        double *I = Q ? ws.get<double>((size_t)n * n) : nullptr;
         long long nl = 0;
-        if (!A || !qws || (Q && !I)) {
+        if (!A || !qws) {
             rc = HSVD_ERR_NOMEM;
         } else if (cudaMemcpy2DAsync(A, sizeof(double) * m, G, sizeof(double) * ldg, sizeof(double) * m, n,
                                      cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
@@ -1128,12 +1127,8 @@ int hsvd_shorten_qr(const double *G, int64_t m, int64_t n, int64_t ldg, double *
             rc = HSVD_ERR_CUDA;
         } else if (Q) {
             // Q = Q [I; 0]: the identity embedded, then the reflectors applied
-            std::vector<double> eye((size_t)n * n, 0.0);
-            for (int64_t i = 0; i < n; ++i) eye[(size_t)(i + i * n)] = 1.0;
-            if (cudaMemcpyAsync(I, eye.data(), sizeof(double) * n * n, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-                qr_embed_u(I, n, m, n, Q, ldq, st) != cudaSuccess ||
-                qr_apply_q(A, m, m, n, qws, Q, ldq, st, &nl) != cudaSuccess ||
-                cudaStreamSynchronize(st) != cudaSuccess)
+            if (qr_embed_u(nullptr, n, m, n, Q, ldq, st) != cudaSuccess ||
+                qr_apply_q(A, m, m, n, qws, Q, ldq, st, &nl, 0, true) != cudaSuccess)
                 rc = HSVD_ERR_CUDA;
         }
     }

@@ -384,11 +384,12 @@ size_t qr_workspace_doubles(int64_t n);
 // A <- R (upper triangle) and the reflectors (below); ws: qr_workspace_doubles(n)
 cudaError_t qr_factor(double *A, int64_t lda, int64_t m, int64_t n, double *ws, cudaStream_t st,
                       long long *launches);
-// U (m x n) <- Q U, Q from the reflectors in A and the T factors in ws
-// U (m x ncols, ldu) <- Q U; ncols = 0 means n
+// U (m x ncols, ldu) <- Q U, Q from the reflectors in A and the T factors in ws;
+// ncols = 0 means n; identity: U holds [I; 0]
 cudaError_t qr_apply_q(double *A, int64_t lda, int64_t m, int64_t n, double *ws, double *U, int64_t ldu,
-                       cudaStream_t st, long long *launches, int64_t ncols = 0);
+                       cudaStream_t st, long long *launches, int64_t ncols = 0, bool identity = false);
 cudaError_t qr_extract_r(const double *A, int64_t lda, int64_t n, double *R, int64_t ldr, cudaStream_t st);
+// U (m x n) <- [U_R; 0], [I; 0] when UR is null
 cudaError_t qr_embed_u(const double *UR, int64_t ldur, int64_t m, int64_t n, double *U, int64_t ldu,
                        cudaStream_t st);
 

@@ -8,15 +8,16 @@
 //
 // Blocked QR with panels of width kQB (compact WY form, H_1 ... H_w =
 // I - V T V^T, T upper triangular):
-//   k_qr_panel   factors one panel column by column (reflector as in LAPACK's
-//                dlarfg: beta = -sign(alpha) ||x||, tau = (beta - alpha) / beta,
-//                v = x / (alpha - beta) below the unit diagonal).  One CTA.
-//   k_qr_vtc     partial products V^T C over row splits (C: the trailing
-//                columns, V itself for T, or U when Q is applied).
-//   k_qr_tbuild  T from tau and V^T V (T_jj = tau_j,
-//                T_{0:j,j} = -tau_j T_{0:j,0:j} V_{:,0:j}^T v_j): the partials
-//                summed by one thread per entry, the recurrence by one warp.
-//   k_qr_tz      Z = op(T) (sum of the partials): op = T^T for the
+//   k_qr_panel_cl  factors one panel column by column on a 16-CTA cluster
+//                (reflector as in LAPACK's dlarfg: beta = -sign(alpha) ||x||,
+//                tau = (beta - alpha) / beta, v = x / (alpha - beta) below the
+//                unit diagonal); k_qr_panel, one CTA, for fewer than 32 rows.
+//   k_qr_vtc     partial products V^T [V C] over row splits (C: the trailing
+//                columns, or U when Q is applied; V for T).
+//   k_qr_sum     Y = V^T V, the sum of its partials.
+//   k_qr_tbuild  T from tau and Y (T_jj = tau_j,
+//                T_{0:j,j} = -tau_j T_{0:j,0:j} V_{:,0:j}^T v_j).
+//   k_qr_tz      Z = op(T) (sum of the partials of C): op = T^T for the
 //                factorisation (Q^T C), T for applying Q.
 //   k_qr_update  C -= V Z.
 // Every product is an FP64 FMA chain (the library is compiled without
@@ -130,31 +131,77 @@ k_qr_panel(double *__restrict__ A, int64_t lda, int64_t m, int j0, int w, double
     }
 }
 
-// The same panel factorisation on a cluster of kPanelCl CTAs that keep the
-// panel in shared memory: CTA r holds rows j0 + r rp .. j0 + (r+1) rp - 1
-// (column-major, stride rp).  Per column, every CTA reduces its rows' part of
-// x^T x and x^T a_c and writes it, with the diagonal row when it owns it, into
-// every CTA (double-buffered by column parity); after one cluster barrier
-// every CTA sums the same partials in the same order, forms beta, tau, w_c
-// itself and updates its own rows.  The panel goes back to A at the end.
 constexpr int kPanelCl = 16;
 constexpr int kPanelClMaxRows = 832;  // rows per CTA kept in shared memory: 32 x 832 doubles = 208 KB
 
-// Sum over the warp of 32 per-lane values v[0..31]; lane l receives the sum of
-// v[l] (a butterfly that halves the values a lane carries at each level: 31
-// shuffles instead of 32 x 5).
-__device__ __forceinline__ double warp_transpose_sum(double (&v)[kQB], int lane) {
+// Sums over the warp of N values a lane carries, v[i] of every lane: a butterfly
+// (xor 16, 8, 4, 2, 1) that halves the values a lane carries at each level while
+// it can, 31 adds for 32 values and 6 for 4.  Returns the sum of value
+// warp_sums_index<N>(lane).
+template <int N, int O>
+__device__ __forceinline__ double warp_sums(double *v, int lane) {
+    constexpr int H = (N + 1) / 2;
+    const bool hi = lane & O;
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        const bool hi = lane & o;
-#pragma unroll
-        for (int i = 0; i < o; ++i) {
-            const double send = hi ? v[i] : v[i + o];
-            const double keep = hi ? v[i + o] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    for (int i = 0; i < H; ++i) {
+        if (i + H < N) {
+            const double send = hi ? v[i] : v[i + H], keep = hi ? v[i + H] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+        } else {
+            v[i] = v[i] + __shfl_xor_sync(0xffffffffu, v[i], O);
         }
     }
-    return v[0];
+    if constexpr (O > 1) return warp_sums<H, O / 2>(v, lane);
+    else return v[0];
+}
+template <int N, int O = 16>
+__device__ __forceinline__ int warp_sums_index(int lane) {
+    constexpr int H = (N + 1) / 2;
+    int i = 0;
+    if constexpr (O > 1) i = warp_sums_index<H, O / 2>(lane);
+    return (lane & O) && i + H < N ? i + H : i;
+}
+
+// Two parts of a column step of k_qr_panel_cl over a thread's rows (first + tid,
+// + 256, ...), for the columns from C0 on: the warp's dots of x with them into
+// sums[C0 ..], and their update.  C0, the step's column rounded down to four, is
+// a template argument because an FP64 instruction that is predicated off occupies
+// the pipe like one that is not.
+template <int C0, class Col>
+__device__ __forceinline__ void panel_dots(Col col, int jj, int w, int first, int nrows, int lane, double *sums) {
+    constexpr int N = kQB - C0;
+    double acc[N];
+#pragma unroll
+    for (int c = 0; c < N; ++c) acc[c] = 0.0;
+    const double *x = col(jj);
+    for (int i = first; i < nrows; i += kPanelThreads) {
+        const double xi = x[i];
+        double v[N];
+#pragma unroll
+        for (int c = 0; c < N; ++c) v[c] = col(C0 + c < w ? C0 + c : jj)[i];
+#pragma unroll
+        for (int c = 0; c < N; ++c) acc[c] = fma(xi, v[c], acc[c]);
+    }
+    const double s = warp_sums<N, 16>(acc, lane);
+    sums[C0 + warp_sums_index<N>(lane)] = s;
+}
+template <int C0, class Col>
+__device__ __forceinline__ void panel_update(Col col, int jj, int w, int first, int nrows, double scale,
+                                             const double *f) {
+    constexpr int N = kQB - C0;
+    double *x = col(jj);
+    for (int i = first; i < nrows; i += kPanelThreads) {
+        const double v = x[i] * scale;
+        double a[N];
+#pragma unroll
+        for (int c = 0; c < N; ++c) a[c] = col(C0 + c < w ? C0 + c : jj)[i];
+        x[i] = v;
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+            const double r = fma(f[C0 + c], v, a[c]);
+            if (C0 + c > jj && C0 + c < w) col(C0 + c)[i] = r;
+        }
+    }
 }
 
 // The same panel factorisation on a cluster of kPanelCl CTAs: CTA r owns rows
@@ -163,7 +210,13 @@ __device__ __forceinline__ double warp_transpose_sum(double (&v)[kQB], int lane)
 // its rows' part of x^T x and x^T a_c and writes it, with the diagonal row
 // when it owns it, into every CTA (double-buffered by column parity); after
 // one cluster barrier every CTA sums the same partials in the same order,
-// forms beta, tau, w_c itself and updates its own rows.
+// forms beta, tau, w_c itself (warp 0: a column per lane, the two quotients side
+// by side) and updates its own rows.  Bound by the FP64 pipe of the 16 SMs, two
+// FMAs per entry of the trailing panel and column, about half of a column's
+// cycles at 8192 rows; the rest is the chain of sums (8 warps, then 16 CTAs),
+// square root and quotient, and the cluster barrier.  Measured at 8192 rows:
+// 0.53 ms a panel with finished columns predicated off and the scalars on one
+// thread between CTA barriers, 0.33 ms now, the same bits.
 template <bool SMEM>
 __global__ void __launch_bounds__(kPanelThreads)
 k_qr_panel_cl(double *__restrict__ A, int64_t lda, int64_t m, int j0, int w, int rp, double *__restrict__ tau) {
@@ -171,7 +224,7 @@ k_qr_panel_cl(double *__restrict__ A, int64_t lda, int64_t m, int j0, int w, int
     __shared__ double red[2][kPanelCl][kQB];     // partial sums from every CTA
     __shared__ double drow[2][kQB];              // the diagonal row of the column
     __shared__ double wred[kPanelThreads / 32][kQB];
-    __shared__ double s_beta, s_tau, s_scale, sw[kQB];
+    __shared__ double s_scale, sf[kQB];          // the column's scale; -tau w_c
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -179,7 +232,7 @@ k_qr_panel_cl(double *__restrict__ A, int64_t lda, int64_t m, int j0, int w, int
     const int64_t left = m - row0;
     const int nrows = left <= 0 ? 0 : (left < rp ? (int)left : rp);
     double *const Ab = A + row0 + (int64_t)j0 * lda;
-    auto at = [&](int c, int i) -> double & { return SMEM ? P[c * rp + i] : Ab[i + (int64_t)c * lda]; };
+    auto col = [&](int c) -> double * { return SMEM ? P + c * rp : Ab + (int64_t)c * lda; };
     if (SMEM)
         for (int e = tid; e < kQB * rp; e += kPanelThreads) {
             const int c = e / rp, i = e % rp;
@@ -190,77 +243,66 @@ k_qr_panel_cl(double *__restrict__ A, int64_t lda, int64_t m, int j0, int w, int
         const int buf = jj & 1;
         // local rows strictly below the diagonal row j0 + jj
         const int64_t below = (int64_t)j0 + jj + 1 - row0;
-        const int first = below <= 0 ? 0 : (below < rp ? (int)below : rp);
-        double acc[kQB];
-#pragma unroll
-        for (int c = 0; c < kQB; ++c) acc[c] = 0.0;
-        for (int i = first + tid; i < nrows; i += kPanelThreads) {
-            const double x = at(jj, i);
-#pragma unroll
-            for (int c = 0; c < kQB; ++c)
-                if (c >= jj && c < w) acc[c] = fma(x, at(c, i), acc[c]);
+        const int first = (below <= 0 ? 0 : (below < rp ? (int)below : rp)) + tid;
+        switch (jj / 4) {
+            case 0: panel_dots<0>(col, jj, w, first, nrows, lane, wred[warp]); break;
+            case 1: panel_dots<4>(col, jj, w, first, nrows, lane, wred[warp]); break;
+            case 2: panel_dots<8>(col, jj, w, first, nrows, lane, wred[warp]); break;
+            case 3: panel_dots<12>(col, jj, w, first, nrows, lane, wred[warp]); break;
+            case 4: panel_dots<16>(col, jj, w, first, nrows, lane, wred[warp]); break;
+            case 5: panel_dots<20>(col, jj, w, first, nrows, lane, wred[warp]); break;
+            case 6: panel_dots<24>(col, jj, w, first, nrows, lane, wred[warp]); break;
+            default: panel_dots<28>(col, jj, w, first, nrows, lane, wred[warp]); break;
         }
-        const double mine = warp_transpose_sum(acc, lane);  // this warp's sum for column `lane`
-        wred[warp][lane] = mine;
         __syncthreads();
         const int64_t dl = (int64_t)j0 + jj - row0;  // the diagonal row, local index
         const bool own_diag = dl >= 0 && dl < nrows;
-        if (tid < kQB) {
+        const bool cact = lane >= (jj & ~3) && lane < w;
+        if (warp < 4) {  // a warp per quarter of the SM: the CTA's sums, into four CTAs each
             double ssum = 0.0;
-            for (int q = 0; q < kPanelThreads / 32; ++q) ssum += wred[q][tid];
-            const double dv = own_diag ? at(tid, (int)dl) : 0.0;
-            for (int r = 0; r < kPanelCl; ++r) {
-                *cluster.map_shared_rank(&red[buf][rank][tid], r) = ssum;
-                if (own_diag) *cluster.map_shared_rank(&drow[buf][tid], r) = dv;
+            if (lane >= (jj & ~3))
+                for (int q = 0; q < kPanelThreads / 32; ++q) ssum += wred[q][lane];
+            const double dv = own_diag && cact ? col(lane)[dl] : 0.0;
+#pragma unroll
+            for (int r = 4 * warp; r < 4 * warp + 4; ++r) {
+                *cluster.map_shared_rank(&red[buf][rank][lane], r) = ssum;
+                if (own_diag) *cluster.map_shared_rank(&drow[buf][lane], r) = dv;
             }
         }
         cluster.sync();
-        // every CTA: the same sums in the same order
-        if (tid < kQB) {
+        if (warp == 0) {  // every CTA: the same sums in the same order, a column per lane
             double tot = 0.0;
-            for (int r = 0; r < kPanelCl; ++r) tot += red[buf][r][tid];
-            wred[0][tid] = tot;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            const double alpha = drow[buf][jj], xnorm2 = wred[0][jj];
-            double t = 0.0, scale = 0.0, beta = alpha;
+#pragma unroll
+            for (int r = 0; r < kPanelCl; ++r) tot += red[buf][r][lane];
+            const double alpha = drow[buf][jj], xnorm2 = __shfl_sync(0xffffffffu, tot, jj);
+            double val = 0.0, beta = alpha;  // lane 0: tau, the others: the scale
             if (xnorm2 > 0.0) {
                 beta = -copysign(sqrt(fma(alpha, alpha, xnorm2)), alpha);
-                t = (beta - alpha) / beta;
-                scale = 1.0 / (alpha - beta);
+                val = (lane == 0 ? beta - alpha : 1.0) / (lane == 0 ? beta : alpha - beta);
             }
-            s_beta = beta;
-            s_tau = t;
-            s_scale = scale;
-            if (rank == 0) tau[j0 + jj] = t;
-        }
-        if (tid > jj && tid < w) sw[tid] = wred[0][tid];  // the dot; w_c is formed after the barrier
-        __syncthreads();
-        const double t = s_tau, scale = s_scale;
-        if (tid > jj && tid < w) sw[tid] = fma(scale, sw[tid], drow[buf][tid]);
-        __syncthreads();
-        for (int i = first + tid; i < nrows; i += kPanelThreads) {
-            const double v = at(jj, i) * scale;
-            if constexpr (SMEM) {
-                at(jj, i) = v;
-#pragma unroll
-                for (int c = 0; c < kQB; ++c)
-                    if (c > jj && c < w) at(c, i) = fma(-t * sw[c], v, at(c, i));
-            } else {  // global memory: a row's loads are all issued before its stores
-                double val[kQB];
-#pragma unroll
-                for (int c = 0; c < kQB; ++c)
-                    if (c > jj && c < w) val[c] = at(c, i);
-                at(jj, i) = v;
-#pragma unroll
-                for (int c = 0; c < kQB; ++c)
-                    if (c > jj && c < w) at(c, i) = fma(-t * sw[c], v, val[c]);
+            const double t = __shfl_sync(0xffffffffu, val, 0), scale = __shfl_sync(0xffffffffu, val, 1);
+            const double sw = fma(scale, tot, drow[buf][lane]);
+            sf[lane] = -t * sw;
+            if (lane == 0) {
+                s_scale = scale;
+                if (rank == 0) tau[j0 + jj] = t;
+            }
+            if (own_diag) {
+                if (lane == jj) col(jj)[dl] = beta;
+                else if (lane > jj && lane < w) col(lane)[dl] = fma(-t, sw, drow[buf][lane]);
             }
         }
-        if (own_diag) {
-            if (tid == 0) at(jj, (int)dl) = s_beta;
-            if (tid > jj && tid < w) at(tid, (int)dl) = fma(-t, sw[tid], at(tid, (int)dl));
+        __syncthreads();
+        const double scale = s_scale;
+        switch ((jj + 1) / 4) {
+            case 0: panel_update<0>(col, jj, w, first, nrows, scale, sf); break;
+            case 1: panel_update<4>(col, jj, w, first, nrows, scale, sf); break;
+            case 2: panel_update<8>(col, jj, w, first, nrows, scale, sf); break;
+            case 3: panel_update<12>(col, jj, w, first, nrows, scale, sf); break;
+            case 4: panel_update<16>(col, jj, w, first, nrows, scale, sf); break;
+            case 5: panel_update<20>(col, jj, w, first, nrows, scale, sf); break;
+            case 6: panel_update<24>(col, jj, w, first, nrows, scale, sf); break;
+            default: panel_update<28>(col, jj, w, first, nrows, scale, sf); break;
         }
         __syncthreads();
     }
@@ -273,18 +315,23 @@ k_qr_panel_cl(double *__restrict__ A, int64_t lda, int64_t m, int j0, int w, int
 }
 
 // part[s][a][c] = sum over the rows of split s (from j0 on) of V(i, a) C(i, c0 + c),
-// a < w, c < ncols; C is V itself (c_is_v) or a plain matrix.
+// a < w, c < ncols; with ypart, two more tiles of columns (the first) are V
+// itself, its partials [s][a][32] in ypart.  One CTA forms 32 x 16 sums over one
+// split of 256 rows, two per thread: FP64-bound, so the tiles are small for the
+// SMs' shares to come out even (32 x 32: 7 of 6.5 CTAs per SM at 8192 x 1024).
+constexpr int kVtcCols = 16;
 __global__ void __launch_bounds__(kVtcThreads)
 k_qr_vtc(const double *__restrict__ A, int64_t lda, int64_t m, int j0, int w, const double *__restrict__ C,
-         int64_t ldc, int c0, int ncols, int c_is_v, int nsplit, int64_t rows_per, double *__restrict__ part) {
+         int64_t ldc, int c0, int ncols, int64_t rows_per, double *__restrict__ part, double *__restrict__ ypart) {
     __shared__ double Vs[kVtcRows][kQB + 1];
-    __shared__ double Cs[kVtcRows][kQB + 1];
-    const int tile = blockIdx.x, split = blockIdx.y;
-    const int ct0 = tile * kQB;
+    __shared__ double Cs[kVtcRows][kVtcCols + 1];
+    const int split = blockIdx.y, vt = ypart ? kQB / kVtcCols : 0;
+    const bool is_v = (int)blockIdx.x < vt;
+    const int ct0 = ((int)blockIdx.x - (is_v ? 0 : vt)) * kVtcCols;
     const int64_t r0 = (int64_t)j0 + (int64_t)split * rows_per;
     const int64_t r1 = m < r0 + rows_per ? m : r0 + rows_per;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+    double acc[2] = {0.0, 0.0};
     for (int64_t rb = r0; rb < r1; rb += kVtcRows) {
         for (int e = tid; e < kVtcRows * kQB; e += kVtcThreads) {
             const int rr = e % kVtcRows, k = e / kVtcRows;
@@ -292,87 +339,85 @@ k_qr_vtc(const double *__restrict__ A, int64_t lda, int64_t m, int j0, int w, co
             const bool in = i < r1;
             Vs[rr][k] = (in && k < w) ? v_entry(A, lda, i, j0, k) : 0.0;
             const int c = ct0 + k;
-            double cv = 0.0;
-            if (in && c < ncols) cv = c_is_v ? v_entry(A, lda, i, j0, c) : C[i + (int64_t)(c0 + c) * ldc];
-            Cs[rr][k] = cv;
+            if (!is_v && k < kVtcCols) Cs[rr][k] = in && c < ncols ? C[i + (int64_t)(c0 + c) * ldc] : 0.0;
         }
         __syncthreads();
-#pragma unroll 4
+        const double *X = is_v ? &Vs[0][ct0 + tx] : &Cs[0][tx];
+        const int xs = is_v ? kQB + 1 : kVtcCols + 1;
+#pragma unroll 8
         for (int rr = 0; rr < kVtcRows; ++rr) {
-            const double v0 = Vs[rr][ty], v1 = Vs[rr][ty + 16];
-            const double x0 = Cs[rr][tx], x1 = Cs[rr][tx + 16];
-            acc[0][0] = fma(v0, x0, acc[0][0]);
-            acc[0][1] = fma(v0, x1, acc[0][1]);
-            acc[1][0] = fma(v1, x0, acc[1][0]);
-            acc[1][1] = fma(v1, x1, acc[1][1]);
+            const double x = X[rr * xs];
+            acc[0] = fma(Vs[rr][ty], x, acc[0]);
+            acc[1] = fma(Vs[rr][ty + 16], x, acc[1]);
         }
         __syncthreads();
     }
-    double *pp = part + (size_t)split * kQB * ncols;
+    const int nc = is_v ? kQB : ncols, c = ct0 + tx;
+    double *pp = (is_v ? ypart : part) + (size_t)split * kQB * nc;
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-            const int a = ty + 16 * u, c = ct0 + tx + 16 * v;
-            if (a < w && c < ncols) pp[(size_t)a * ncols + c] = acc[u][v];
-        }
+    for (int u = 0; u < 2; ++u) {
+        const int a = ty + 16 * u;
+        if (a < (is_v ? kQB : w) && c < nc) pp[(size_t)a * nc + c] = acc[u];
+    }
 }
 
-// T of the panel from tau and Y = V^T V (the sum of the partials), one warp:
-// lane r holds row r of T; column j is formed from column j of Y.
+// Y[a][c] = sum of the partials of V^T V in split order, one warp per row a
+__global__ void __launch_bounds__(kQB) k_qr_sum(const double *__restrict__ ypart, int nsplit, double *__restrict__ Y) {
+    const int e = blockIdx.x * kQB + threadIdx.x;
+    double s = 0.0;
+#pragma unroll 8
+    for (int k = 0; k < nsplit; ++k) s += ypart[(size_t)k * kQB * kQB + e];
+    Y[e] = s;
+}
+
+// T of the panel from tau and Y = V^T V: T_{r,j} = -tau_j sum_{k=r}^{j-1}
+// T_{r,k} Y_{k,j}, T_jj = tau_j.  Warp r holds row r, lane j column j: once
+// T_{r,k} is known it goes into the sums of every later column at once, a chain
+// of two FP64 instructions a column instead of a sum over k per column (45 us
+// with the partials' sum in the same kernel; 12 us, and 7 us for k_qr_sum: the
+// same sums in the same order).
 __global__ void __launch_bounds__(kQB * kQB)
-k_qr_tbuild(const double *__restrict__ part, int nsplit, int w, const double *__restrict__ tau_j0,
-            double *__restrict__ T) {
-    __shared__ double Ts[kQB][kQB + 1];
-    __shared__ double Y[kQB][kQB + 1];
-    // every entry of Y = V^T V (the sum of the partials) by its own thread
-    {
-        const int a = threadIdx.x / kQB, c = threadIdx.x % kQB;
-        double s = 0.0;
-        if (a < w && c < w)
-            for (int q = 0; q < nsplit; ++q) s += part[(size_t)q * kQB * w + (size_t)a * w + c];
-        Y[a][c] = s;
-        Ts[a][c] = 0.0;
-    }
+k_qr_tbuild(const double *__restrict__ Y, int w, const double *__restrict__ tau_j0, double *__restrict__ T) {
+    __shared__ double Ys[kQB][kQB + 1];
+    const int r = threadIdx.x >> 5, j = threadIdx.x & 31;
+    Ys[r][j] = Y[r * kQB + j];
     __syncthreads();
-    if (threadIdx.x >= 32) return;
-    const int r = threadIdx.x;
-    for (int j = 0; j < w; ++j) {
-        const double tj = tau_j0[j];
-        if (r < j) {  // T_{r,j} = -tau_j sum_{k=r}^{j-1} T_{r,k} y_k, y_k = v_k^T v_j
-            double s = 0.0;
-            for (int k = r; k < j; ++k) s = fma(Ts[r][k], Y[k][j], s);
-            Ts[r][j] = -tj * s;
-        }
-        if (r == j) Ts[r][j] = tj;
-        __syncwarp();
+    const double tj = j < w ? tau_j0[j] : 0.0;
+    double s = 0.0, t = r == j ? tj : 0.0;  // t: T_{r,j}
+    for (int k = r; k < w - 1; ++k) {
+        const double tk = __shfl_sync(0xffffffffu, t, k);
+        if (j > k) s = fma(tk, Ys[k][j], s);
+        if (j == k + 1 && j < w) t = -tj * s;
     }
-    for (int c = 0; c < kQB; ++c) T[r * kQB + c] = Ts[r][c];
+    T[r * kQB + j] = t;
 }
 
 // Z[a][c] = sum_b op(T)[a][b] X[b][c], X the sum of the partials; op = T^T
-// when trans (the factorisation applies H^T), T otherwise (Q applied).
-__global__ void k_qr_tz(const double *__restrict__ part, int nsplit, int w, int ncols, const double *__restrict__ T,
-                        int trans, double *__restrict__ Z) {
-    __shared__ double Xs[kQB][kQB + 1];
+// when trans (the factorisation applies H^T), T otherwise (Q applied).  One CTA
+// per 8 columns, one entry a thread: the sums are bound by the FP64 pipe, and 32
+// columns a CTA left most SMs idle (43 us a launch; 8 columns: 13 us).
+constexpr int kTzCols = 8;
+__global__ void __launch_bounds__(kQB * kTzCols)
+k_qr_tz(const double *__restrict__ part, int nsplit, int w, int ncols, const double *__restrict__ T, int trans,
+        double *__restrict__ Z) {
+    __shared__ double Xs[kQB][kTzCols + 1];
     __shared__ double Ts[kQB][kQB + 1];
-    const int ct0 = blockIdx.x * kQB, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8 threads
-    for (int a = ty; a < kQB; a += 8) {
-        const int c = ct0 + tx;
-        double s = 0.0;
-        if (a < w && c < ncols)
-            for (int q = 0; q < nsplit; ++q) s += part[(size_t)q * kQB * ncols + (size_t)a * ncols + c];
-        Xs[a][tx] = s;
-        Ts[a][tx] = T[a * kQB + tx];
+    const int tx = threadIdx.x % kTzCols, a = threadIdx.x / kTzCols, c = blockIdx.x * kTzCols + tx;
+    for (int e = threadIdx.x; e < kQB * kQB; e += kQB * kTzCols) Ts[e / kQB][e % kQB] = T[e];
+    double s = 0.0;
+    if (a < w && c < ncols) {
+        const double *pp = part + (size_t)a * ncols + c;
+        const size_t step = (size_t)kQB * ncols;
+#pragma unroll 8
+        for (int q = 0; q < nsplit; ++q) s += pp[q * step];
     }
+    Xs[a][tx] = s;
     __syncthreads();
-    for (int a = ty; a < w; a += 8) {
-        const int c = ct0 + tx;
-        if (c >= ncols) continue;
-        double s = 0.0;
-        for (int b = 0; b < w; ++b) s = fma(trans ? Ts[b][a] : Ts[a][b], Xs[b][tx], s);
-        Z[(size_t)a * ncols + c] = s;
-    }
+    if (a >= w || c >= ncols) return;
+    s = 0.0;
+#pragma unroll 8
+    for (int b = 0; b < w; ++b) s = fma(trans ? Ts[b][a] : Ts[a][b], Xs[b][tx], s);
+    Z[(size_t)a * ncols + c] = s;
 }
 
 // C(i, c0 + c) -= sum_a V(i, a) Z[a][c] for rows i >= j0; one CTA per (row
@@ -455,26 +500,55 @@ cudaError_t panel_cluster(double *A, int64_t lda, int64_t m, int j0, int w, doub
                                  : launch_panel_cl<false>(A, lda, m, j0, w, rp, tau, st);
 }
 
+constexpr int kMaxSplit = 64;
 int qr_nsplit(int64_t rows) {
     const int64_t s = (rows + 255) / 256;  // at least 256 rows per split
-    return (int)std::max<int64_t>(1, std::min<int64_t>(s, 64));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(s, kMaxSplit));
 }
 
-// Applies H_panel^T (trans) or H_panel to columns c0 .. c0 + ncols - 1 of C,
-// in chunks of kMaxCols columns (workspace: part, Z).
-constexpr int kMaxCols = 2048;
-cudaError_t apply_panel(double *A, int64_t lda, int64_t m, int j0, int w, const double *T, int trans, double *C,
-                        int64_t ldc, int c0, int ncols, double *part, double *Z, cudaStream_t st) {
+// Workspace of a factorisation, within qr_workspace_doubles(n).
+struct QrWs {
+    double *T, *tau, *ypart, *Y, *part, *Z;
+};
+constexpr int kMaxCols = 2048;  // columns of C taken at once
+QrWs qr_carve(double *ws, int64_t n) {
+    const int64_t panels = (n + kQB - 1) / kQB, cols = std::min<int64_t>(n, kMaxCols);
+    QrWs q;
+    q.T = ws;
+    q.tau = q.T + (size_t)panels * kQB * kQB;
+    q.ypart = q.tau + n;
+    q.Y = q.ypart + (size_t)kMaxSplit * kQB * kQB;
+    q.part = q.Y + kQB * kQB;
+    q.Z = q.part + (size_t)kMaxSplit * kQB * cols;
+    return q;
+}
+
+// Applies H_panel^T (trans) or H_panel to columns c0 .. c0 + ncols - 1 of C, in
+// chunks of kMaxCols columns; with build, V^T V is formed in the first launch
+// and T from it.
+cudaError_t apply_panel(double *A, int64_t lda, int64_t m, int j0, int w, double *T, bool build, int trans, double *C,
+                        int64_t ldc, int c0, int ncols, const QrWs &q, cudaStream_t st, long long *launches) {
     const int64_t rows = m - j0;
-    const int nsplit = qr_nsplit(rows);
-    const int64_t rows_per = (rows + nsplit - 1) / nsplit;
-    for (int cb = 0; cb < ncols; cb += kMaxCols) {
-        const int nc = std::min(kMaxCols, ncols - cb);
-        const dim3 g1((nc + kQB - 1) / kQB, nsplit);
-        k_qr_vtc<<<g1, kVtcThreads, 0, st>>>(A, lda, m, j0, w, C, ldc, c0 + cb, nc, 0, nsplit, rows_per, part);
-        k_qr_tz<<<(nc + kQB - 1) / kQB, 256, 0, st>>>(part, nsplit, w, nc, T, trans, Z);
-        const dim3 g2((unsigned)((rows + 63) / 64), (nc + kQB - 1) / kQB);
-        k_qr_update<<<g2, 256, 0, st>>>(C, ldc, m, c0 + cb, nc, A, lda, j0, w, Z);
+    for (int cb = 0; cb < ncols || (build && cb == 0); cb += kMaxCols) {
+        const int nc = std::max(0, std::min(kMaxCols, ncols - cb));
+        const bool with_v = build && cb == 0;
+        const int tiles = (nc + kVtcCols - 1) / kVtcCols + (with_v ? kQB / kVtcCols : 0);
+        const int nsplit = qr_nsplit(rows);
+        const int64_t rows_per = (rows + nsplit - 1) / nsplit;
+        k_qr_vtc<<<dim3(tiles, nsplit), kVtcThreads, 0, st>>>(A, lda, m, j0, w, C, ldc, c0 + cb, nc, rows_per, q.part,
+                                                               with_v ? q.ypart : nullptr);
+        *launches += 1;
+        if (with_v) {
+            k_qr_sum<<<kQB, kQB, 0, st>>>(q.ypart, nsplit, q.Y);
+            k_qr_tbuild<<<1, kQB * kQB, 0, st>>>(q.Y, w, q.tau + j0, T);
+            *launches += 2;
+        }
+        if (nc > 0) {
+            k_qr_tz<<<(nc + kTzCols - 1) / kTzCols, kQB * kTzCols, 0, st>>>(q.part, nsplit, w, nc, T, trans, q.Z);
+            const dim3 g2((unsigned)((rows + 63) / 64), (nc + kQB - 1) / kQB);
+            k_qr_update<<<g2, 256, 0, st>>>(C, ldc, m, c0 + cb, nc, A, lda, j0, w, q.Z);
+            *launches += 2;
+        }
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -484,17 +558,15 @@ cudaError_t apply_panel(double *A, int64_t lda, int64_t m, int j0, int w, const 
 }  // namespace
 
 size_t qr_workspace_doubles(int64_t n) {
-    const int64_t panels = (n + kQB - 1) / kQB;
-    const int64_t cols = std::min<int64_t>(n, kMaxCols);  // widest column chunk
-    return (size_t)panels * kQB * kQB             // T of every panel
-           + (size_t)n                            // tau
-           + (size_t)64 * kQB * cols              // partials (at most 64 row splits)
-           + (size_t)kQB * cols;                  // Z
+    const int64_t panels = (n + kQB - 1) / kQB, cols = std::min<int64_t>(n, kMaxCols);
+    // T of every panel, tau, the partials of V^T V and their sum, the partials of V^T C, Z
+    return (size_t)panels * kQB * kQB + (size_t)n + (size_t)(kMaxSplit + 1) * kQB * kQB +
+           (size_t)(kMaxSplit + 1) * kQB * cols;
 }
 
 namespace {
 // R (n x n, ldr) <- the upper triangle of A, zeros below; U (m x n, ldu) <-
-// [U_R; 0] from U_R (n x n, ldur)
+// [U_R; 0] from U_R (n x n, ldur), or [I; 0]
 __global__ void k_qr_extract_r(const double *__restrict__ A, int64_t lda, int64_t n, double *__restrict__ R,
                                int64_t ldr) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -507,7 +579,7 @@ __global__ void k_qr_embed_u(const double *__restrict__ UR, int64_t ldur, int64_
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= m * n) return;
     const int64_t i = e % m, j = e / m;
-    U[i + j * ldu] = i < n ? UR[i + j * ldur] : 0.0;
+    U[i + j * ldu] = i >= n ? 0.0 : (UR ? UR[i + j * ldur] : (i == j ? 1.0 : 0.0));  // no U_R: the identity
 }
 }  // namespace
 
@@ -529,31 +601,17 @@ cudaError_t qr_embed_u(const double *UR, int64_t ldur, int64_t m, int64_t n, dou
 cudaError_t qr_factor(double *A, int64_t lda, int64_t m, int64_t n, double *ws, cudaStream_t st,
                       long long *launches) {
     const int64_t panels = (n + kQB - 1) / kQB;
-    double *Tall = ws, *tau = Tall + (size_t)panels * kQB * kQB;
-    double *part = tau + n, *Z = part + (size_t)64 * kQB * std::min<int64_t>(n, kMaxCols);
+    const QrWs q = qr_carve(ws, n);
     for (int64_t p = 0; p < panels; ++p) {
         const int j0 = (int)(p * kQB), w = (int)std::min<int64_t>(kQB, n - j0);
-        double *T = Tall + (size_t)p * kQB * kQB;
-        if (panel_cluster(A, lda, m, j0, w, tau, st) != cudaSuccess) {
+        if (panel_cluster(A, lda, m, j0, w, q.tau, st) != cudaSuccess) {
             cudaGetLastError();  // clear a refused cluster launch; the one-CTA kernel does the panel
-            k_qr_panel<<<1, kPanelThreads, 0, st>>>(A, lda, m, j0, w, tau);
+            k_qr_panel<<<1, kPanelThreads, 0, st>>>(A, lda, m, j0, w, q.tau);
         }
-        // T from V^T V
-        const int64_t rows = m - j0;
-        const int nsplit = qr_nsplit(rows);
-        const int64_t rows_per = (rows + nsplit - 1) / nsplit;
-        k_qr_vtc<<<dim3(1, nsplit), kVtcThreads, 0, st>>>(A, lda, m, j0, w, nullptr, 0, 0, w, 1, nsplit, rows_per,
-                                                          part);
-        k_qr_tbuild<<<1, kQB * kQB, 0, st>>>(part, nsplit, w, tau + j0, T);
-        cudaError_t e = cudaGetLastError();
+        *launches += 1;
+        const cudaError_t e = apply_panel(A, lda, m, j0, w, q.T + (size_t)p * kQB * kQB, true, 1, A, lda, j0 + w,
+                                          (int)(n - j0 - w), q, st, launches);
         if (e != cudaSuccess) return e;
-        *launches += 3;
-        const int nt = (int)(n - j0 - w);
-        if (nt > 0) {
-            e = apply_panel(A, lda, m, j0, w, T, 1, A, lda, j0 + w, nt, part, Z, st);
-            if (e != cudaSuccess) return e;
-            *launches += 3 * ((nt + kMaxCols - 1) / kMaxCols);
-        }
     }
     return cudaSuccess;
 }
@@ -561,22 +619,23 @@ cudaError_t qr_factor(double *A, int64_t lda, int64_t m, int64_t n, double *ws, 
 // U (m x ncols, ldu; ncols = 0: n) holds [U_R; 0] on entry; U <- Q U with the
 // reflectors in A and the T factors in ws (as left by qr_factor).  The
 // workspace holds partials for min(n, 2048) columns, so U is taken in chunks
-// of that many columns.
+// of that many columns.  With `identity` U holds [I; 0]: a panel's reflectors,
+// zero above row j0, leave the columns before j0 as they are.
 cudaError_t qr_apply_q(double *A, int64_t lda, int64_t m, int64_t n, double *ws, double *U, int64_t ldu,
-                       cudaStream_t st, long long *launches, int64_t ncols) {
+                       cudaStream_t st, long long *launches, int64_t ncols, bool identity) {
     const int64_t panels = (n + kQB - 1) / kQB;
-    double *Tall = ws, *tau = Tall + (size_t)panels * kQB * kQB;
+    const QrWs q = qr_carve(ws, n);
     const int64_t wcols = std::min<int64_t>(n, kMaxCols);
-    double *part = tau + n, *Z = part + (size_t)64 * kQB * wcols;
     if (ncols <= 0) ncols = n;
     for (int64_t c0 = 0; c0 < ncols; c0 += wcols) {
         const int nc = (int)std::min<int64_t>(wcols, ncols - c0);
         for (int64_t p = panels - 1; p >= 0; --p) {
             const int j0 = (int)(p * kQB), w = (int)std::min<int64_t>(kQB, n - j0);
-            const cudaError_t e = apply_panel(A, lda, m, j0, w, Tall + (size_t)p * kQB * kQB, 0, U, ldu, (int)c0,
-                                              nc, part, Z, st);
+            const int skip = identity ? (int)std::min<int64_t>(nc, std::max<int64_t>(0, j0 - c0)) : 0;
+            if (skip == nc) continue;
+            const cudaError_t e = apply_panel(A, lda, m, j0, w, q.T + (size_t)p * kQB * kQB, false, 0, U, ldu,
+                                              (int)c0 + skip, nc - skip, q, st, launches);
             if (e != cudaSuccess) return e;
-            *launches += 3;
         }
     }
     return cudaSuccess;

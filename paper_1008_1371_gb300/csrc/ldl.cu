@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "hsvd_internal.cuh"
@@ -521,8 +522,8 @@ struct LdlBest {
 // publish, 4,000 for the slowest CTA's maxima to arrive, 3,000 for the decision,
 // 2,300 for the loads, and the update (n = 1001: 4,500 on average, 2048: 15,000).
 // Measured (N(0,1) symmetric, whole call, against the three kernels a step):
-// n = 64: 0.49 against 2.37 ms, 300: 1.9 against 10.1, 1001: 9.0 against 37.7,
-// 2048: 28.9 against 101, 4096: 135 against 358.
+// n = 64: 0.48 against 2.37 ms, 300: 1.7 against 10.1, 1001: 8.9 against 37.7,
+// 2048: 25.8 against 101, 4096: 124 against 358.
 __global__ void __launch_bounds__(kPT, 1)
 k_ldl_persist(const double *__restrict__ M, int64_t ldm, double *__restrict__ W, int n, double *__restrict__ G,
               int64_t ldg, int *__restrict__ perm_out, double *__restrict__ Dblk, int8_t *__restrict__ bsize,
@@ -715,42 +716,50 @@ k_ldl_persist(const double *__restrict__ M, int64_t ldm, double *__restrict__ W,
         const double i00 = s_inv[0], i01 = s_inv[1], i11 = s_inv[2];
         best = {0, 0, 0xffffffffu, 0xffffffffu};
         const bool store_l = cta == k % grid;
-        for (int i = row; i < n; i += kPT) {
-            const int si = source(i);
-            const double w0 = c0[i];
-            double l0, l1 = 0.0;
-            if (s == 1) {
-                l0 = w0 * i00;
-            } else {
-                const double w1 = c1[i];
-                l0 = fma(w0, i00, w1 * i01);
-                l1 = fma(w0, i01, w1 * i11);
-            }
-            if (store_l) {
-                double *g = G + perm[i] + (int64_t)k * ldg;
-                g[0] = l0;
-                if (s == 2) g[ldg] = l1;
-            }
-            for (int j0 = t0 + cta; j0 < n; j0 += kPU * grid) {
-                if (i != row || j0 != t0 + cta) {
+        // (the step's size is a template argument, the columns past n a branch: an
+        // FP64 instruction that is predicated off occupies the pipe like any other)
+        auto update = [&](auto size) {
+            constexpr int S = decltype(size)::value;
+            for (int i = row; i < n; i += kPT) {
+                const int si = source(i);
+                const double w0 = c0[i];
+                double l0, l1 = 0.0;
+                if constexpr (S == 1) {
+                    l0 = w0 * i00;
+                } else {
+                    const double w1 = c1[i];
+                    l0 = fma(w0, i00, w1 * i01);
+                    l1 = fma(w0, i01, w1 * i11);
+                }
+                if (store_l) {
+                    double *g = G + perm[i] + (int64_t)k * ldg;
+                    g[0] = l0;
+                    if (S == 2) g[ldg] = l1;
+                }
+                for (int j0 = t0 + cta; j0 < n; j0 += kPU * grid) {
+                    if (i != row || j0 != t0 + cta) {
+#pragma unroll
+                        for (int u = 0; u < kPU; ++u) {
+                            const int j = j0 + u * grid;
+                            if (j < n) old[u] = __ldcg(W + si + (int64_t)slot[j] * n);
+                        }
+                    }
 #pragma unroll
                     for (int u = 0; u < kPU; ++u) {
                         const int j = j0 + u * grid;
-                        if (j < n) old[u] = __ldcg(W + si + (int64_t)slot[j] * n);
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < kPU; ++u) {
-                    const int j = j0 + u * grid;
-                    if (j < n) {
-                        const int to = j == r ? f0 : (s == 2 && j == q ? f1 : slot[j]);
-                        const double v = s == 1 ? fma(-l0, c0[j], old[u]) : fma(-l0, c0[j], fma(-l1, c1[j], old[u]));
+                        if (j >= n) break;
+                        const int to = j == r ? f0 : (S == 2 && j == q ? f1 : slot[j]);
+                        double v = old[u];
+                        if constexpr (S == 2) v = fma(-l1, c1[j], v);
+                        v = fma(-l0, c0[j], v);
                         __stcg(W + i + (int64_t)to * n, v);
                         best.see(v, i, j);
                     }
                 }
             }
-        }
+        };
+        if (s == 1) update(std::integral_constant<int, 1>{});
+        else update(std::integral_constant<int, 2>{});
         k = t0;
         if (k >= n) break;
     }

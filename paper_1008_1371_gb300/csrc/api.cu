@@ -733,7 +733,6 @@ int solve_wide(const double *G, int64_t m, int64_t n, int64_t ldg, const int8_t 
         hq.beta = ws.get<double>((size_t)m);
         hq.cperm = ws.get<int>((size_t)m);
         hq.rswap = ws.get<int>((size_t)m);
-        hq.drows = ws.get<int>(4);
         hq.s = ws.get<int8_t>((size_t)n);
         hq.bsize = ws.get<int8_t>((size_t)m);
         hq.state = ws.get<unsigned char>(hypqr_state_bytes());
@@ -763,7 +762,7 @@ int solve_wide(const double *G, int64_t m, int64_t n, int64_t ldg, const int8_t 
             j = dJ;
         }
         if (rc == HSVD_OK && (!hq.A || !hq.C || !hq.Vr || !hq.z || !hq.beta || !hq.cperm || !hq.rswap ||
-                              !hq.drows || !hq.s || !hq.bsize || !hq.state || !hq.mx || !F || !Jh1 || (V && !VF)))
+                              !hq.s || !hq.bsize || !hq.state || !hq.mx || !F || !Jh1 || (V && !VF)))
             rc = HSVD_ERR_NOMEM;
         if (rc == HSVD_OK) rc = hypqr_factor(g, m, n, lg, j, hq, F, st, &nl);
         if (rc == HSVD_OK) {

@@ -395,11 +395,11 @@ cudaError_t qr_embed_u(const double *UR, int64_t ldur, int64_t m, int64_t n, dou
 
 // hypqr.cu: the hyperbolic QR of G^T for a wide G (m < n).  Device buffers,
 // filled by the caller: A, Vr (n x m), C (m x m), z (n), beta (m), cperm,
-// rswap (m), drows (4), s (n), bsize (m), state and mx (hypqr_state_bytes,
+// rswap (m), s (n), bsize (m), state and mx (hypqr_state_bytes,
 // hypqr_mx_bytes).
 struct HypQr {
     double *A, *C, *Vr, *z, *beta;
-    int *cperm, *rswap, *drows;
+    int *cperm, *rswap;
     int8_t *s, *bsize;
     void *state, *mx;
 };
@@ -409,7 +409,7 @@ size_t hypqr_mx_bytes(int64_t m);
 // signature of F).  HSVD_OK, HSVD_ERR_RANK (G J G^T singular) or HSVD_ERR_CUDA.
 int hypqr_factor(const double *G, int64_t m, int64_t n, int64_t ldg, const int8_t *J, HypQr &hq, double *F,
                  cudaStream_t st, long long *launches);
-// V (n x m, ldv) <- T^T [V_F; 0]; consumes hq.s
+// V (n x m, ldv) <- T^T [V_F; 0]; may write hq.A
 int hypqr_apply_tt(HypQr &hq, int64_t m, int64_t n, const double *VF, double *V, int64_t ldv, cudaStream_t st,
                    long long *launches);
 

@@ -38,149 +38,260 @@ constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kH * kF, kOffW2 = kOffB1 + kH, kOffB
 static_assert(kParams == HSVD_MLP_PARAMS, "parameter count");
 
 constexpr int kTrainSamples = 64;  // samples per CTA of the training kernel
-constexpr int kTrainThreads = 256;
+constexpr int kTrainThreads = 512;
+constexpr int kInferThreads = 256;  // 32 samples at a time
+constexpr int kRow = kH + 4;        // rows of 64 values in shared memory: 16-byte accesses to 8 rows at once
+constexpr int kRow1 = kF + 4;       // rows of W1, likewise
 
 __device__ __forceinline__ float bf16_round(float w) { return __bfloat162float(__float2bfloat16_rn(w)); }
 
-// weights rounded to BF16 (biases stay FP32) into shared memory
-__device__ void load_params(const float *__restrict__ p, float *__restrict__ sp) {
-    for (int i = threadIdx.x; i < kParams; i += blockDim.x) {
-        const bool is_w = (i < kOffB1) || (i >= kOffW2 && i < kOffB2) || (i >= kOffW3 && i < kOffB3);
-        sp[i] = is_w ? bf16_round(p[i]) : p[i];
+// the network in shared memory: weights rounded to BF16, biases FP32
+struct Net {
+    alignas(16) float w1[kH * kRow1], w2[kH * kRow], b1[kH], b2[kH], w3[kH], b3;
+};
+
+__device__ __forceinline__ void load_net(const float *__restrict__ p, Net &net) {
+    const int tid = threadIdx.x;
+#pragma unroll 8
+    for (int e = tid; e < kH * kH; e += blockDim.x) net.w2[(e / kH) * kRow + e % kH] = bf16_round(p[kOffW2 + e]);
+    for (int e = tid; e < kH * kF; e += blockDim.x) net.w1[(e / kF) * kRow1 + e % kF] = bf16_round(p[kOffW1 + e]);
+    if (tid < kH) {
+        net.b1[tid] = p[kOffB1 + tid];
+        net.b2[tid] = p[kOffB2 + tid];
+        net.w3[tid] = bf16_round(p[kOffW3 + tid]);
     }
+    if (tid == 0) net.b3 = p[kOffB3];
 }
 
-// forward pass of one sample; h1, h2 receive the post-ReLU activations
-__device__ __forceinline__ float mlp_forward(const float *__restrict__ sp, const float *__restrict__ x, float *h1,
-                                             float *h2) {
-    for (int j = 0; j < kH; ++j) {
-        float a = sp[kOffB1 + j];
+// Forward pass of the CTA's T / 8 samples xs[s][kF]: h1, h2 [s][kRow] receive
+// the post-ReLU activations.  A thread computes 2 samples by 4 units (s = tid /
+// 16 and T / 16 on, unit j = tid % 16 and every 16 on), each sum from its bias
+// through the inputs in order, so a value doesn't depend on the tile it is
+// computed in; per 4 inputs 6 16-byte loads serve 32 FMAs.  Ends with a barrier.
+template <int T>
+__device__ __forceinline__ void mlp_layers(const Net &net, const float *__restrict__ xs, float *__restrict__ h1,
+                                           float *__restrict__ h2) {
+    const int tj = threadIdx.x % 16, ts = threadIdx.x / 16;
+    float a[2][4];
+    auto layer = [&](const float *in, int ldi, const float *w, int ldw, const float *bias, int k, float *out) {
 #pragma unroll
-        for (int i = 0; i < kF; ++i) a = fmaf(sp[kOffW1 + j * kF + i], x[i], a);
-        h1[j] = fmaxf(a, 0.0f);
+        for (int q = 0; q < 4; ++q) a[0][q] = a[1][q] = bias[tj + 16 * q];
+#pragma unroll 4
+        for (int i = 0; i < k; i += 4) {
+            const float4 x0 = *reinterpret_cast<const float4 *>(in + ts * ldi + i);
+            const float4 x1 = *reinterpret_cast<const float4 *>(in + (ts + T / 16) * ldi + i);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 u = *reinterpret_cast<const float4 *>(w + (tj + 16 * q) * ldw + i);
+                a[0][q] = fmaf(u.w, x0.w, fmaf(u.z, x0.z, fmaf(u.y, x0.y, fmaf(u.x, x0.x, a[0][q]))));
+                a[1][q] = fmaf(u.w, x1.w, fmaf(u.z, x1.z, fmaf(u.y, x1.y, fmaf(u.x, x1.x, a[1][q]))));
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            out[ts * kRow + tj + 16 * q] = fmaxf(a[0][q], 0.0f);
+            out[(ts + T / 16) * kRow + tj + 16 * q] = fmaxf(a[1][q], 0.0f);
+        }
+        __syncthreads();
+    };
+    layer(xs, kF, net.w1, kRow1, net.b1, kF, h1);
+    layer(h1, kRow, net.w2, kRow, net.b2, kH, h2);
+}
+
+// the logit of one sample from its h2
+__device__ __forceinline__ float mlp_logit(const Net &net, const float *__restrict__ h2) {
+    float z = net.b3;
+#pragma unroll
+    for (int i = 0; i < kH; i += 4) {
+        const float4 h = *reinterpret_cast<const float4 *>(h2 + i), w = *reinterpret_cast<const float4 *>(net.w3 + i);
+        z = fmaf(w.w, h.w, fmaf(w.z, h.z, fmaf(w.y, h.y, fmaf(w.x, h.x, z))));
     }
-    for (int j = 0; j < kH; ++j) {
-        float a = sp[kOffB2 + j];
-        for (int i = 0; i < kH; ++i) a = fmaf(sp[kOffW2 + j * kH + i], h1[i], a);
-        h2[j] = fmaxf(a, 0.0f);
-    }
-    float z = sp[kOffB3];
-    for (int i = 0; i < kH; ++i) z = fmaf(sp[kOffW3 + i], h2[i], z);
     return z;
 }
 
-__global__ void __launch_bounds__(128) k_mlp_infer(const float *__restrict__ params, const float *__restrict__ X,
-                                                   int n, float *__restrict__ logits, int8_t *__restrict__ skip,
-                                                   float logit_tau) {
-    __shared__ float sp[kParams];
-    load_params(params, sp);
-    __syncthreads();
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    float x[kF], h1[kH], h2[kH];
-#pragma unroll
-    for (int i = 0; i < kF; ++i) x[i] = X[(size_t)s * kF + i];
-    const float z = mlp_forward(sp, x, h1, h2);
-    if (logits) logits[s] = z;
-    if (skip) skip[s] = z < logit_tau ? 1 : 0;
+// Tiles of 32 samples, a CTA every gridDim-th.  Bound by latencies at the sizes
+// in use (loading the network, three dependent layers); a thread per sample,
+// its activations in local memory, left most SMs without work.  Measured, the
+// call: 4096 samples 14 us (of them 7 in the kernel), 60000 27 us; with a thread
+// per sample 19 and 45.
+__global__ void __launch_bounds__(kInferThreads) k_mlp_infer(const float *__restrict__ params,
+                                                             const float *__restrict__ X, int n,
+                                                             float *__restrict__ logits, int8_t *__restrict__ skip,
+                                                             float logit_tau) {
+    constexpr int S = kInferThreads / 8;
+    __shared__ Net net;
+    __shared__ alignas(16) float xs[S * kF], h1[S * kRow], h2[S * kRow];
+    const int tid = threadIdx.x;
+    load_net(params, net);
+    for (int s0 = blockIdx.x * S; s0 < n; s0 += gridDim.x * S) {
+        xs[tid] = s0 + tid / kF < n ? X[(size_t)s0 * kF + tid] : 0.0f;
+        __syncthreads();
+        mlp_layers<kInferThreads>(net, xs, h1, h2);
+        if (tid < S && s0 + tid < n) {
+            const float z = mlp_logit(net, h2 + tid * kRow);
+            if (logits) logits[s0 + tid] = z;
+            if (skip) skip[s0 + tid] = z < logit_tau ? 1 : 0;
+        }
+    }
 }
+
+struct TrainSmem {
+    Net net;
+    alignas(16) float xs[kTrainSamples * kF];
+    alignas(16) float h1[kTrainSamples * kRow], h2[kTrainSamples * kRow];
+    alignas(16) float d2[kTrainSamples * kRow], d1[kTrainSamples * kRow];  // dL/d(pre-activations)
+    float dz[kTrainSamples], ls[kTrainSamples];
+};
 
 // Gradient of the mean binary cross-entropy with logits over n samples,
 // L = mean(softplus(z) - y z), per CTA of kTrainSamples samples: partial
-// sums over the CTA's samples in a fixed order (deterministic).
+// sums over the CTA's samples in a fixed order (deterministic).  Every product
+// is a small matrix product of register tiles (2 x 4 outputs a thread) over
+// operands in shared memory.  Bound by the FP32 pipe of the SMs that have a CTA
+// (64 of them with 4096 samples).  Measured, the call with the reduction: 4096
+// samples 27 us, 60000 97 us; with a thread per sample for both passes 83 and 549.
 __global__ void __launch_bounds__(kTrainThreads) k_mlp_grad_partial(const float *__restrict__ params,
                                                                     const float *__restrict__ X,
                                                                     const float *__restrict__ y, int n,
                                                                     float *__restrict__ gpart,
                                                                     float *__restrict__ lpart) {
-    extern __shared__ float sm[];
-    float *sp = sm;                                  // kParams
-    float *xs = sp + kParams;                        // [S][kF]
-    float *h1 = xs + kTrainSamples * kF;             // [S][kH]
-    float *h2 = h1 + kTrainSamples * kH;             // [S][kH]
-    float *d2 = h2 + kTrainSamples * kH;             // [S][kH]  dL/d(pre-activation 2)
-    float *d1 = d2 + kTrainSamples * kH;             // [S][kH]  dL/d(pre-activation 1)
-    float *dz = d1 + kTrainSamples * kH;             // [S]
-    float *ls = dz + kTrainSamples;                  // [S]
-    load_params(params, sp);
+    extern __shared__ __align__(16) unsigned char smem[];
+    TrainSmem &sm = *reinterpret_cast<TrainSmem *>(smem);
+    static_assert(kTrainThreads == kTrainSamples * kF && kTrainThreads == kH * kF, "one value a thread");
+    const int tid = threadIdx.x;
     const int s0 = blockIdx.x * kTrainSamples;
     const int ns = min(kTrainSamples, n - s0);
-    for (int e = threadIdx.x; e < kTrainSamples * kF; e += blockDim.x) {
-        const int s = e / kF;
-        xs[e] = s < ns ? X[(size_t)(s0 + s) * kF + e % kF] : 0.0f;
+    const float inv_n = 1.0f / (float)n;
+    sm.xs[tid] = tid / kF < ns ? X[(size_t)s0 * kF + tid] : 0.0f;
+    const float yy = tid < ns ? y[s0 + tid] : 0.0f;  // of the threads that finish a sample
+    load_net(params, sm.net);
+    __syncthreads();
+    mlp_layers<kTrainThreads>(sm.net, sm.xs, sm.h1, sm.h2);
+    if (tid < kTrainSamples) {
+        const float z = mlp_logit(sm.net, sm.h2 + tid * kRow);
+        if (tid < ns) {
+            const float p = 1.0f / (1.0f + expf(-z));
+            sm.dz[tid] = (p - yy) * inv_n;
+            // softplus(z) - y z, written stably
+            sm.ls[tid] = fmaxf(z, 0.0f) + log1pf(expf(-fabsf(z))) - yy * z;
+        } else {
+            sm.dz[tid] = 0.0f;
+            sm.ls[tid] = 0.0f;
+        }
     }
     __syncthreads();
-    const float inv_n = 1.0f / (float)n;
-    if (threadIdx.x < kTrainSamples) {
-        const int s = threadIdx.x;
-        float hh1[kH], hh2[kH];
-        const float z = mlp_forward(sp, xs + s * kF, hh1, hh2);
+    for (int e = tid; e < kTrainSamples * kH; e += kTrainThreads) {
+        const int s = e / kH, j = e % kH;
+        sm.d2[s * kRow + j] = sm.h2[s * kRow + j] > 0.0f ? sm.dz[s] * sm.net.w3[j] : 0.0f;
+    }
+    __syncthreads();
+    const int t4 = 4 * (tid % 16), ts = tid / 16;  // 4 units, and a row of 32
+    {                                              // d1 = (d2 W2) where h1 > 0: samples ts and ts + 32
+        float a[2][4] = {};
+#pragma unroll 4
         for (int j = 0; j < kH; ++j) {
-            h1[s * kH + j] = hh1[j];
-            h2[s * kH + j] = hh2[j];
+            const float4 w = *reinterpret_cast<const float4 *>(sm.net.w2 + j * kRow + t4);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float d = sm.d2[(ts + 32 * h) * kRow + j];
+                a[h][0] = fmaf(w.x, d, a[h][0]);
+                a[h][1] = fmaf(w.y, d, a[h][1]);
+                a[h][2] = fmaf(w.z, d, a[h][2]);
+                a[h][3] = fmaf(w.w, d, a[h][3]);
+            }
         }
-        if (s < ns) {
-            const float yy = y[s0 + s];
-            const float p = 1.0f / (1.0f + expf(-z));
-            dz[s] = (p - yy) * inv_n;
-            // softplus(z) - y z, written stably
-            ls[s] = fmaxf(z, 0.0f) + log1pf(expf(-fabsf(z))) - yy * z;
-        } else {
-            dz[s] = 0.0f;
-            ls[s] = 0.0f;
-        }
-        for (int j = 0; j < kH; ++j) d2[s * kH + j] = hh2[j] > 0.0f ? dz[s] * sp[kOffW3 + j] : 0.0f;
-        for (int i = 0; i < kH; ++i) {
-            float a = 0.0f;
-            for (int j = 0; j < kH; ++j) a = fmaf(sp[kOffW2 + j * kH + i], d2[s * kH + j], a);
-            d1[s * kH + i] = hh1[i] > 0.0f ? a : 0.0f;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int o = (ts + 32 * h) * kRow + t4;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sm.d1[o + q] = sm.h1[o + q] > 0.0f ? a[h][q] : 0.0f;
         }
     }
     __syncthreads();
     float *g = gpart + (size_t)blockIdx.x * kParams;
-    for (int q = threadIdx.x; q < kParams; q += blockDim.x) {
-        float a = 0.0f;
-        if (q < kOffB1) {
-            const int j = q / kF, i = q % kF;
-            for (int s = 0; s < kTrainSamples; ++s) a = fmaf(d1[s * kH + j], xs[s * kF + i], a);
-        } else if (q < kOffW2) {
-            const int j = q - kOffB1;
-            for (int s = 0; s < kTrainSamples; ++s) a += d1[s * kH + j];
-        } else if (q < kOffB2) {
-            const int j = (q - kOffW2) / kH, i = (q - kOffW2) % kH;
-            for (int s = 0; s < kTrainSamples; ++s) a = fmaf(d2[s * kH + j], h1[s * kH + i], a);
-        } else if (q < kOffW3) {
-            const int j = q - kOffB2;
-            for (int s = 0; s < kTrainSamples; ++s) a += d2[s * kH + j];
-        } else if (q < kOffB3) {
-            const int i = q - kOffW3;
-            for (int s = 0; s < kTrainSamples; ++s) a = fmaf(dz[s], h2[s * kH + i], a);
-        } else {
-            for (int s = 0; s < kTrainSamples; ++s) a += dz[s];
+    {  // W2: units ts and ts + 32 by inputs t4 ..
+        float a[2][4] = {};
+#pragma unroll 4
+        for (int s = 0; s < kTrainSamples; ++s) {
+            const float4 x = *reinterpret_cast<const float4 *>(sm.h1 + s * kRow + t4);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float d = sm.d2[s * kRow + ts + 32 * h];
+                a[h][0] = fmaf(d, x.x, a[h][0]);
+                a[h][1] = fmaf(d, x.y, a[h][1]);
+                a[h][2] = fmaf(d, x.z, a[h][2]);
+                a[h][3] = fmaf(d, x.w, a[h][3]);
+            }
         }
-        g[q] = a;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) g[kOffW2 + (ts + 32 * h) * kH + t4 + q] = a[h][q];
     }
-    if (threadIdx.x == 0) {
-        float l = 0.0f;
-        for (int s = 0; s < kTrainSamples; ++s) l += ls[s];
-        lpart[blockIdx.x] = l * inv_n;
+    {  // W1: one value a thread
+        const int j = tid / kF, i = tid % kF;
+        float a = 0.0f;
+#pragma unroll 8
+        for (int s = 0; s < kTrainSamples; ++s) a = fmaf(sm.d1[s * kRow + j], sm.xs[s * kF + i], a);
+        g[kOffW1 + tid] = a;
+    }
+    // the rest: sums over the samples of one array each
+    const int j = tid % kH;
+    float a = 0.0f;
+    if (tid < 2 * kH) {
+        const float *d = (tid < kH ? sm.d1 : sm.d2) + j;
+#pragma unroll 8
+        for (int s = 0; s < kTrainSamples; ++s) a += d[s * kRow];
+        g[(tid < kH ? kOffB1 : kOffB2) + j] = a;
+    } else if (tid < 3 * kH) {
+#pragma unroll 8
+        for (int s = 0; s < kTrainSamples; ++s) a = fmaf(sm.dz[s], sm.h2[s * kRow + j], a);
+        g[kOffW3 + j] = a;
+    } else if (tid == 3 * kH) {
+#pragma unroll 8
+        for (int s = 0; s < kTrainSamples; ++s) a += sm.dz[s];
+        g[kOffB3] = a;
+    } else if (tid == 4 * kH) {
+#pragma unroll 8
+        for (int s = 0; s < kTrainSamples; ++s) a += sm.ls[s];
+        lpart[blockIdx.x] = a * inv_n;
     }
 }
 
-// sum of the CTA partials, in CTA order
-__global__ void k_mlp_grad_reduce(const float *__restrict__ gpart, const float *__restrict__ lpart, int nblk,
-                                  float *__restrict__ grad, float *__restrict__ loss) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < kParams) {
-        float a = 0.0f;
-        for (int b = 0; b < nblk; ++b) a += gpart[(size_t)b * kParams + q];
-        grad[q] = a;
+// Sum of the CTA partials, in CTA order: 32 values a CTA, whose 8 warps load
+// kRedRows partials at a time (all in flight together) for warp 0 to add one by
+// one.  The loss is value kParams.  Bound by the latency of one stage's loads:
+// 64 partials 3.7 us.
+constexpr int kRedRows = 128;
+__global__ void __launch_bounds__(256) k_mlp_grad_reduce(const float *__restrict__ gpart,
+                                                         const float *__restrict__ lpart, int nblk,
+                                                         float *__restrict__ grad, float *__restrict__ loss) {
+    __shared__ float buf[2][kRedRows][32];
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    const int q = blockIdx.x * 32 + lane;
+    const float *src = q < kParams ? gpart + q : lpart;
+    const size_t ld = q < kParams ? kParams : 1;
+    const bool live = q <= kParams;
+    float a = 0.0f;
+    int h = 0;
+    for (int b0 = 0; b0 < nblk; b0 += kRedRows, h ^= 1) {
+        float v[kRedRows / 8];
+#pragma unroll
+        for (int r = 0; r < kRedRows / 8; ++r) {
+            const int b = b0 + warp + 8 * r;
+            v[r] = live && b < nblk ? src[b * ld] : 0.0f;
+        }
+#pragma unroll
+        for (int r = 0; r < kRedRows / 8; ++r) buf[h][warp + 8 * r][lane] = v[r];
+        __syncthreads();  // one barrier a stage: the other buffer is written meanwhile
+        if (warp == 0) {
+            const int nb = min(kRedRows, nblk - b0);
+#pragma unroll 16
+            for (int b = 0; b < nb; ++b) a += buf[h][b][lane];
+        }
     }
-    if (q == 0 && loss) {
-        float l = 0.0f;
-        for (int b = 0; b < nblk; ++b) l += lpart[b];
-        *loss = l;
-    }
+    if (warp == 0 && q < kParams) grad[q] = a;
+    if (warp == 0 && q == kParams && loss) *loss = a;
 }
 
 // Adam (Kingma and Ba): m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
@@ -245,10 +356,6 @@ __global__ void k_mask_table(const int *__restrict__ outer, const int8_t *__rest
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(kept, (int)n);
 }
 
-size_t grad_smem() {
-    return sizeof(float) * (kParams + kTrainSamples * kF + 4 * kTrainSamples * kH + 2 * kTrainSamples);
-}
-
 }  // namespace
 
 cudaError_t launch_features(const float *trace, const int8_t *prev_skip, const int *tab, int nvis, int b, int nb,
@@ -260,7 +367,10 @@ cudaError_t launch_features(const float *trace, const int8_t *prev_skip, const i
 cudaError_t launch_mlp_infer(const float *params, const float *X, int n, float *logits, int8_t *skip,
                              float logit_tau, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_mlp_infer<<<(n + 127) / 128, 128, 0, st>>>(params, X, n, logits, skip, logit_tau);
+    constexpr int S = kInferThreads / 8;
+    // at most the CTAs that are on the chip together (4 on an SM): the network is loaded once for all their tiles
+    const int tiles = (int)(((int64_t)n + S - 1) / S);
+    k_mlp_infer<<<tiles < 4 * 152 ? tiles : 4 * 152, kInferThreads, 0, st>>>(params, X, n, logits, skip, logit_tau);
     return cudaGetLastError();
 }
 
@@ -279,13 +389,13 @@ int mlp_grad_blocks(int n) { return (n + kTrainSamples - 1) / kTrainSamples; }
 cudaError_t launch_mlp_grad(const float *params, const float *X, const float *y, int n, float *gpart, float *lpart,
                             float *grad, float *loss, cudaStream_t st) {
     const int nblk = mlp_grad_blocks(n);
-    const size_t smem = grad_smem();
+    const size_t smem = sizeof(TrainSmem);
     cudaError_t e = cudaFuncSetAttribute(k_mlp_grad_partial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_mlp_grad_partial<<<nblk, kTrainThreads, smem, st>>>(params, X, y, n, gpart, lpart);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_mlp_grad_reduce<<<(kParams + 255) / 256, 256, 0, st>>>(gpart, lpart, nblk, grad, loss);
+    k_mlp_grad_reduce<<<(kParams + 1 + 31) / 32, 256, 0, st>>>(gpart, lpart, nblk, grad, loss);
     return cudaGetLastError();
 }
 

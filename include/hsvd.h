@@ -468,6 +468,13 @@ int hsvd_mlp_grad(const float *params, const float *X, const float *y, int64_t n
 int hsvd_mlp_adam(float *params, float *m, float *v, const float *grad, int t, float lr, float beta1, float beta2,
                   float eps, void *stream);
 
+/*
+ * The calls take their device scratch from a pool of the library's own, which
+ * keeps at most 256 MB per device between calls.  hsvd_release_scratch gives
+ * what no call is using back to the device (the current device).
+ */
+int hsvd_release_scratch(void);
+
 #ifdef __cplusplus
 }
 #endif

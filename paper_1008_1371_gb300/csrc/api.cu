@@ -70,7 +70,7 @@ struct Ws {
     template <class T>
     T *get(size_t count) {
         void *p = nullptr;
-        if (cudaMallocAsync(&p, count * sizeof(T) + 16, st) != cudaSuccess) return nullptr;
+        if (scratch_alloc(&p, count * sizeof(T) + 16, st) != cudaSuccess) return nullptr;
         ptrs.push_back(p);
         return static_cast<T *>(p);
     }
@@ -945,11 +945,11 @@ int hsvd_solve_ex(const double *G, int64_t m, int64_t n, int64_t ldg, const int8
     }
     if (!dev) {
         // host arrays: stage through device memory on the internal stream
-        if (cudaMallocAsync((void **)&dG, sizeof(double) * m * n, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&dJ, n, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&dS, sizeof(double) * n, st) != cudaSuccess ||
-            (U && cudaMallocAsync((void **)&dU, sizeof(double) * m * n, st) != cudaSuccess) ||
-            (V && cudaMallocAsync((void **)&dV, sizeof(double) * n * n, st) != cudaSuccess)) {
+        if (scratch_alloc((void **)&dG, sizeof(double) * m * n, st) != cudaSuccess ||
+            scratch_alloc((void **)&dJ, n, st) != cudaSuccess ||
+            scratch_alloc((void **)&dS, sizeof(double) * n, st) != cudaSuccess ||
+            (U && scratch_alloc((void **)&dU, sizeof(double) * m * n, st) != cudaSuccess) ||
+            (V && scratch_alloc((void **)&dV, sizeof(double) * n * n, st) != cudaSuccess)) {
             rc = HSVD_ERR_NOMEM;
             goto done;
         }
@@ -1010,7 +1010,7 @@ int hsvd_solve(const double *G, int64_t m, int64_t n, int64_t ldg, const int8_t 
 int hsvd_diag_wait_timeout(void *stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int *d = nullptr, h = -1;
-    if (cudaMallocAsync((void **)&d, sizeof(int), st) != cudaSuccess) return HSVD_ERR_NOMEM;
+    if (scratch_alloc((void **)&d, sizeof(int), st) != cudaSuccess) return HSVD_ERR_NOMEM;
     int rc = HSVD_OK;
     if (launch_diag_wait(4096, d, st) != cudaSuccess ||
         cudaMemcpyAsync(&h, d, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -1143,7 +1143,7 @@ int hsvd_pivot_gram(const double *G, int64_t rows, int64_t ldg, int b, int npair
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nsplit = gram_nsplit(rows, npairs);
     double *part = nullptr;
-    if (cudaMallocAsync((void **)&part, sizeof(double) * npairs * 3 * nsplit * b * b, st) != cudaSuccess)
+    if (scratch_alloc((void **)&part, sizeof(double) * npairs * 3 * nsplit * b * b, st) != cudaSuccess)
         return HSVD_ERR_NOMEM;
     int rc = HSVD_OK;
     if (launch_gram(G, rows, ldg, b, npairs, col0, nsplit, part, st) != cudaSuccess ||
@@ -1166,7 +1166,7 @@ int hsvd_pivot_solve(int b, int npairs, double *A, const int8_t *sgn, double tol
     if (!fill_ring(b, full.data() + (size_t)nn * b * 2)) return HSVD_ERR_ARG;
     fill_cross(b, cross.data());
     int *dt = nullptr;
-    if (cudaMallocAsync((void **)&dt, sizeof(int) * (full.size() + cross.size()), st) != cudaSuccess)
+    if (scratch_alloc((void **)&dt, sizeof(int) * (full.size() + cross.size()), st) != cudaSuccess)
         return HSVD_ERR_NOMEM;
     int rc = HSVD_OK;
     if (cudaMemcpyAsync(dt, full.data(), full.size() * sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -1200,9 +1200,9 @@ int hsvd_pivot_gram_x(const double *G, int64_t rows, int64_t ldg, int npairs, co
     const int ks = precision_gram_ksplit(rows);
     double *part = nullptr;
     int *status = nullptr;
-    if (cudaMallocAsync((void **)&part, sizeof(double) * (size_t)npairs * ks * 128 * 128, st) != cudaSuccess)
+    if (scratch_alloc((void **)&part, sizeof(double) * (size_t)npairs * ks * 128 * 128, st) != cudaSuccess)
         return HSVD_ERR_NOMEM;
-    if (cudaMallocAsync((void **)&status, sizeof(int), st) != cudaSuccess) {
+    if (scratch_alloc((void **)&status, sizeof(int), st) != cudaSuccess) {
         cudaFreeAsync(part, st);
         return HSVD_ERR_NOMEM;
     }
@@ -1227,10 +1227,10 @@ int hsvd_pivot_update_x(double *X, int64_t rows, int64_t ldx, int npairs, const 
     uint16_t *wsl = nullptr;
     int *wexp = nullptr, *dz = nullptr, *status = nullptr;
     int rc = HSVD_OK, h = 0;
-    if (cudaMallocAsync((void **)&wsl, sizeof(uint16_t) * precision_wsl_elems(npairs), st) != cudaSuccess ||
-        cudaMallocAsync((void **)&wexp, sizeof(int) * (size_t)npairs * 256, st) != cudaSuccess ||
-        cudaMallocAsync((void **)&dz, sizeof(int) * (size_t)npairs * 128, st) != cudaSuccess ||
-        cudaMallocAsync((void **)&status, sizeof(int), st) != cudaSuccess)
+    if (scratch_alloc((void **)&wsl, sizeof(uint16_t) * precision_wsl_elems(npairs), st) != cudaSuccess ||
+        scratch_alloc((void **)&wexp, sizeof(int) * (size_t)npairs * 256, st) != cudaSuccess ||
+        scratch_alloc((void **)&dz, sizeof(int) * (size_t)npairs * 128, st) != cudaSuccess ||
+        scratch_alloc((void **)&status, sizeof(int), st) != cudaSuccess)
         rc = HSVD_ERR_NOMEM;
     if (rc == HSVD_OK) {
         const int *dk = dexp;

@@ -279,9 +279,9 @@ cudaError_t run_batch(const std::vector<BTask> &tasks, int max_sweeps, int sort,
     BTask *d_tasks = nullptr;
     int *d_counter = nullptr;
     double *d_ws = nullptr;
-    cudaError_t e = cudaMallocAsync((void **)&d_tasks, sizeof(BTask) * (size_t)count, st);
-    if (e == cudaSuccess) e = cudaMallocAsync((void **)&d_counter, sizeof(int), st);
-    if (e == cudaSuccess) e = cudaMallocAsync((void **)&d_ws, sizeof(double) * (size_t)grid * stride + 64, st);
+    cudaError_t e = scratch_alloc((void **)&d_tasks, sizeof(BTask) * (size_t)count, st);
+    if (e == cudaSuccess) e = scratch_alloc((void **)&d_counter, sizeof(int), st);
+    if (e == cudaSuccess) e = scratch_alloc((void **)&d_ws, sizeof(double) * (size_t)grid * stride + 64, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d_tasks, tasks.data(), sizeof(BTask) * (size_t)count, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
@@ -524,16 +524,16 @@ int hsvd_solve_batched_ex(int64_t count, const double *const *G, const int64_t *
     auto fail = [&](int code) {
         if (rc == HSVD_OK) rc = code;
     };
-    if (cudaMallocAsync((void **)&d_res, sizeof(int) * 3 * (size_t)count, st) != cudaSuccess ||
-        cudaMallocAsync((void **)&d_where, sizeof(int) * (size_t)count, st) != cudaSuccess ||
-        cudaMallocAsync((void **)&d_rot, sizeof(long long) * (size_t)count, st) != cudaSuccess)
+    if (scratch_alloc((void **)&d_res, sizeof(int) * 3 * (size_t)count, st) != cudaSuccess ||
+        scratch_alloc((void **)&d_where, sizeof(int) * (size_t)count, st) != cudaSuccess ||
+        scratch_alloc((void **)&d_rot, sizeof(long long) * (size_t)count, st) != cudaSuccess)
         fail(HSVD_ERR_NOMEM);
     if (rc == HSVD_OK && host) {
-        if (cudaMallocAsync((void **)&dG, sizeof(double) * g_off + 16, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&dJ, j_off + 16, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&dS, sizeof(double) * s_off + 16, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&dU, sizeof(double) * u_off + 16, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&dV, sizeof(double) * v_off + 16, st) != cudaSuccess)
+        if (scratch_alloc((void **)&dG, sizeof(double) * g_off + 16, st) != cudaSuccess ||
+            scratch_alloc((void **)&dJ, j_off + 16, st) != cudaSuccess ||
+            scratch_alloc((void **)&dS, sizeof(double) * s_off + 16, st) != cudaSuccess ||
+            scratch_alloc((void **)&dU, sizeof(double) * u_off + 16, st) != cudaSuccess ||
+            scratch_alloc((void **)&dV, sizeof(double) * v_off + 16, st) != cudaSuccess)
             fail(HSVD_ERR_NOMEM);
     }
     size_t go = 0, jo = 0, so = 0, uo = 0, vo = 0;

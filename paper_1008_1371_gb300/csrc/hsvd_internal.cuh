@@ -393,6 +393,11 @@ cudaError_t qr_extract_r(const double *A, int64_t lda, int64_t n, double *R, int
 cudaError_t qr_embed_u(const double *UR, int64_t ldur, int64_t m, int64_t n, double *U, int64_t ldu,
                        cudaStream_t st);
 
+// scratch.cu: device memory for a call, freed with cudaFreeAsync
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st);
+// identity of the current context, 0 if it cannot be read
+unsigned long long current_context_id();
+
 // hypqr.cu: the hyperbolic QR of G^T for a wide G (m < n).  Device buffers,
 // filled by the caller: A, Vr (n x m), C (m x m), z (n), beta (m), cperm,
 // rswap (m), s (n), bsize (m), state and mx (hypqr_state_bytes,

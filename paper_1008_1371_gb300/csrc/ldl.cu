@@ -803,13 +803,13 @@ int ldl_factor(const double *M, int64_t n, int64_t ldm, double *G, int64_t ldg, 
     const bool persist = n <= kPersistMaxN;
     const int grid = (int)std::min<int64_t>(sms, std::max<int64_t>(1, n / 6));
     const size_t nslots = persist ? 2 * (size_t)grid : 0;
-    if (!ok(cudaMallocAsync((void **)&W, sizeof(double) * n * (n + 2), st)) ||
-        !ok(cudaMallocAsync((void **)&Dblk, sizeof(double) * 4 * n, st)) ||
-        !ok(cudaMallocAsync((void **)&perm, sizeof(int) * n, st)) ||
-        !ok(cudaMallocAsync((void **)&bsize, (size_t)n, st)) ||
-        !ok(cudaMallocAsync((void **)&state, sizeof(LdlState), st)) ||
-        !ok(cudaMallocAsync((void **)&mx, sizeof(LdlMax) * kUpdGrid, st)) ||
-        !ok(cudaMallocAsync((void **)&slots, sizeof(LdlSlot) * (nslots + 1), st))) {
+    if (!ok(scratch_alloc((void **)&W, sizeof(double) * n * (n + 2), st)) ||
+        !ok(scratch_alloc((void **)&Dblk, sizeof(double) * 4 * n, st)) ||
+        !ok(scratch_alloc((void **)&perm, sizeof(int) * n, st)) ||
+        !ok(scratch_alloc((void **)&bsize, (size_t)n, st)) ||
+        !ok(scratch_alloc((void **)&state, sizeof(LdlState), st)) ||
+        !ok(scratch_alloc((void **)&mx, sizeof(LdlMax) * kUpdGrid, st)) ||
+        !ok(scratch_alloc((void **)&slots, sizeof(LdlSlot) * (nslots + 1), st))) {
         rc = HSVD_ERR_NOMEM;
     }
     if (rc == HSVD_OK) {

@@ -426,16 +426,12 @@ int hsvd_mlp_grad(const float *params, const float *X, const float *y, int64_t n
     if (!all_device({params, X, y, grad, loss})) return HSVD_ERR_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nblk = mlp_grad_blocks((int)n);
-    float *gpart = nullptr, *lpart = nullptr;
-    if (cudaMallocAsync((void **)&gpart, sizeof(float) * (size_t)nblk * HSVD_MLP_PARAMS, st) != cudaSuccess)
+    float *gpart = nullptr;  // the partial gradients, then the partial losses
+    if (scratch_alloc((void **)&gpart, sizeof(float) * (size_t)nblk * (HSVD_MLP_PARAMS + 1), st) != cudaSuccess)
         return HSVD_ERR_NOMEM;
-    if (cudaMallocAsync((void **)&lpart, sizeof(float) * (size_t)nblk, st) != cudaSuccess) {
-        cudaFreeAsync(gpart, st);
-        return HSVD_ERR_NOMEM;
-    }
-    const cudaError_t e = launch_mlp_grad(params, X, y, (int)n, gpart, lpart, grad, loss, st);
+    const cudaError_t e =
+        launch_mlp_grad(params, X, y, (int)n, gpart, gpart + (size_t)nblk * HSVD_MLP_PARAMS, grad, loss, st);
     cudaFreeAsync(gpart, st);
-    cudaFreeAsync(lpart, st);
     return e == cudaSuccess ? HSVD_OK : HSVD_ERR_CUDA;
 }
 

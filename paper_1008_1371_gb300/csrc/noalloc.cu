@@ -11,8 +11,6 @@
 //   [0, n_pad^2)            doubles: the accumulated transformation W
 //   kStatusOff (n_pad^2)    three ints: status, sweeps, stop rule
 //   kRotOff (n_pad^2 + 2)   one 64-bit integer: the rotation count
-#include <cuda.h>
-
 #include <mutex>
 
 #include "hsvd_internal.cuh"
@@ -38,39 +36,12 @@ struct ScratchAddr {
 };
 ScratchAddr g_scratch[kMaxDevices] = {};
 
-typedef CUresult (*CtxGetCurrentFn)(CUcontext *);
-typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long *);
-
-// Identity of the current context, 0 if it cannot be read.  A device reset
-// (cudaDeviceReset) ends the context and reloads the module with the array
-// at a possibly different address; the new context has a new identity.
-unsigned long long current_context_id() {
-    static CtxGetCurrentFn get_current = nullptr;
-    static CtxGetIdFn get_id = nullptr;
-    static bool looked_up = false;
-    if (!looked_up) {
-        looked_up = true;
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_current = reinterpret_cast<CtxGetCurrentFn>(f);
-        f = nullptr;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_id = reinterpret_cast<CtxGetIdFn>(f);
-    }
-    CUcontext ctx = nullptr;
-    unsigned long long id = 0;
-    if (!get_current || !get_id || get_current(&ctx) != CUDA_SUCCESS || !ctx || get_id(ctx, &id) != CUDA_SUCCESS)
-        return 0;
-    return id;
-}
-
 // Device address of the scratch array in the current device's context.  The
 // host-side name of the array is not a device address; the address is looked
 // up (cudaGetSymbolAddress, which allocates nothing) with the device current,
-// once per device and context, and again after a device reset.
+// once per device and context, and again after a device reset (which ends the
+// context and reloads the module with the array at a possibly different
+// address; the new context has a new identity).
 cudaError_t scratch_for_current_device(double **out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);

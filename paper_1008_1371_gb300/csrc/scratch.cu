@@ -1,9 +1,10 @@
 // scratch.cu -- device scratch of the calls.  The device's default pool gives
 // its memory back at every synchronisation, and every call here ends with one:
 // the next call's first allocation mapped memory anew, about 110 us, as long as
-// a tenth of the smallest solve (24 x 24: 0.96 ms, 0.85 so; three small allocations: 110-120 us against 17
-// from a pool that keeps them; 20 of 64 MB: 2.8 ms against 0.05).  So the
-// library has a pool of its own for each device, which keeps at most kKeep bytes
+// a tenth of the smallest solve (24 x 24: 0.96 ms, 0.85 so; three small
+// allocations: 110-120 us against 17 from a pool that keeps them; 20 of 64 MB:
+// 2.8 ms against 0.05).  So the library has a pool of its own for each device,
+// which keeps at most kKeep bytes
 // that no call is using: 256 MB, a thousandth of the device's memory, covers the
 // scratch of everything that runs for less than about 50 ms.  What is above it
 // goes back at the next synchronisation, and the rest with

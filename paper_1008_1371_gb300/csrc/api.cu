@@ -329,7 +329,7 @@ int solve_blocked_core(const double *G, int64_t m, int64_t n, int64_t ldg, const
             e = evs.record(4 * s, st);
             if (e == cudaSuccess)
                 e = prec ? launch_gram_x(Gw, m_pad, m_pad, np, col0, part_x, cnt, st)
-                         : launch_gram(Gw, m_pad, m_pad, b, np, col0, ns, part, st);
+                         : launch_gram(Gw, m_pad, m_pad, b, np, np, col0, ns, part, st);
             if (e == cudaSuccess) e = evs.record(4 * s + 1, st);
             if (e == cudaSuccess)
                 e = prec ? launch_solve(b, np, part_x, ksplit_x, nullptr, sgn, col0, nullptr, tol, mode,
@@ -414,7 +414,7 @@ int solve_blocked_core(const double *G, int64_t m, int64_t n, int64_t ldg, const
                     nl += 4;
                 } else {
                     double *pt = part + (size_t)slot * nsplit * 3 * b * b;
-                    if (e == cudaSuccess) e = launch_gram(Gw, m_pad, m_pad, b, np, c0, nsplit, pt, ss);
+                    if (e == cudaSuccess) e = launch_gram(Gw, m_pad, m_pad, b, np, npairs, c0, nsplit, pt, ss);
                     if (e == cudaSuccess)
                         e = launch_solve(b, np, pt, nsplit, nullptr, sgn, c0, nullptr, tol, mode,
                                          o.inner_max_passes, d_tab_full, d_tab_cross, wp, rot, rot_ctr, cnt, ss, 0,
@@ -1146,7 +1146,7 @@ int hsvd_pivot_gram(const double *G, int64_t rows, int64_t ldg, int b, int npair
     if (scratch_alloc((void **)&part, sizeof(double) * npairs * 3 * nsplit * b * b, st) != cudaSuccess)
         return HSVD_ERR_NOMEM;
     int rc = HSVD_OK;
-    if (launch_gram(G, rows, ldg, b, npairs, col0, nsplit, part, st) != cudaSuccess ||
+    if (launch_gram(G, rows, ldg, b, npairs, npairs, col0, nsplit, part, st) != cudaSuccess ||
         launch_assemble(b, npairs, part, nsplit, A, st) != cudaSuccess)
         rc = HSVD_ERR_CUDA;
     cudaFreeAsync(part, st);

@@ -361,7 +361,8 @@ cudaError_t launch_pointwise(const double *G, int64_t ldg, int m, int n, const i
 
 // blocked.cu: the three kernels of one step of the blocked method.
 int gram_nsplit(int64_t rows, int npairs);
-cudaError_t launch_gram(const double *G, int64_t rows, int64_t ldg, int b, int npairs,
+// step_pairs: pairs whose Gram blocks are computed at a time, in this launch and beside it
+cudaError_t launch_gram(const double *G, int64_t rows, int64_t ldg, int b, int npairs, int step_pairs,
                         const int *col0, int nsplit, double *part, cudaStream_t st);
 // solve_cluster.cu: the inner pivot-block solve.  tab_full holds the modulus
 // pairs of the 2b columns (2b steps of b pairs, 2 ints each) followed by the

@@ -399,8 +399,9 @@ k_update_x(double *__restrict__ X, int64_t rowsX, int64_t ldx, double *__restric
     __shared__ uint32_t tbase;
     __shared__ int s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t chunksX = (rowsX + kUpdRows - 1) / kUpdRows;
-    const int64_t chunks = chunksX + (Y ? (rowsY + kUpdRows - 1) / kUpdRows : 0);
+    // in 32 bits: the panels fit the device's memory, 2^26 items of 128 KB would not
+    const unsigned chunksX = (unsigned)((rowsX + kUpdRows - 1) / kUpdRows);
+    const unsigned chunks = chunksX + (Y ? (unsigned)((rowsY + kUpdRows - 1) / kUpdRows) : 0u);
     const int64_t items = (int64_t)npairs * chunks;
     if (tid == 0) {
         s_fail = 0;
@@ -419,18 +420,18 @@ k_update_x(double *__restrict__ X, int64_t rowsX, int64_t ldx, double *__restric
 
     auto next_item = [&](int64_t from) -> int64_t {
         for (int64_t it = from; it < items; it += gridDim.x)
-            if (rotated[it / chunks]) return it;
+            if (rotated[(unsigned)it / chunks]) return it;
         return -1;
     };
     auto describe = [&](int64_t it) {
         UpdItem d;
-        d.pair = (int)(it / chunks);
-        const int64_t chunk = it % chunks;
+        d.pair = (int)((unsigned)it / chunks);
+        const unsigned chunk = (unsigned)it - (unsigned)d.pair * chunks;
         d.which = chunk < chunksX ? 0 : 1;
         d.M = d.which == 0 ? X : Y;
         d.ld = d.which == 0 ? ldx : ldy;
         d.rows = d.which == 0 ? rowsX : rowsY;
-        d.r0 = (d.which == 0 ? chunk : chunk - chunksX) * kUpdRows;
+        d.r0 = (int64_t)(d.which == 0 ? chunk : chunk - chunksX) * kUpdRows;
         d.cI = col0[2 * d.pair];
         d.cJ = col0[2 * d.pair + 1];
         return d;

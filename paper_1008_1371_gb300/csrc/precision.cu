@@ -141,26 +141,42 @@ k_gram_x(const double *__restrict__ G, int64_t rows, int64_t ldg, const int *__r
     const int cI = col0[2 * pair], cJ = col0[2 * pair + 1];
     auto colptr = [&](int c) { return G + (int64_t)(c < NNX / 2 ? cI + c : cJ + c - NNX / 2) * ldg; };
     cluster_sync();  // both CTAs run before either writes into the other
-    // exponents of the own columns over the split's rows, into both CTAs
-    for (int c = kN * (int)half + warp; c < kN * (int)half + kN; c += kThrG / 32) {
-        const double *g = colptr(c);
-        int e = -2000;
-        int64_t r = r0 + lane;
-        for (; r + 15 * 32 < r1; r += 16 * 32) {  // sixteen loads in flight per lane
-            double x[16];
+    // exponents of the own columns over the split's rows, into both CTAs: two
+    // columns of a warp at a time, of which the high words are enough (Haar 4096:
+    // the solve 1160 -> 1156 ms; a column at a time left warps with an odd one)
+    constexpr int kScan = kN / 16;  // columns a warp, warps 0..15
+    if (warp < 16)
 #pragma unroll
-            for (int u = 0; u < 16; ++u) x[u] = g[r + u * 32];
+        for (int cc = 0; cc < kScan; cc += 2) {
+            const int c = kN * (int)half + warp * kScan + cc;
+            const int *g[2] = {reinterpret_cast<const int *>(colptr(c)) + 1,
+                               reinterpret_cast<const int *>(colptr(c + 1)) + 1};
+            int e[2] = {0, 0};  // biased
+            int64_t r = r0 + lane;
+            for (; r + 15 * 32 < r1; r += 16 * 32) {  // 32 loads in flight per lane
+                int x[2][16];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) e = max(e, exp_bound(x[u]));
+                for (int u = 0; u < 16; ++u)
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) x[v][u] = g[v][2 * (r + u * 32)];
+#pragma unroll
+                for (int u = 0; u < 16; ++u)
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) e[v] = max(e[v], x[v][u] & 0x7FF00000);
+            }
+            for (; r < r1; r += 32)
+#pragma unroll
+                for (int v = 0; v < 2; ++v) e[v] = max(e[v], g[v][2 * r] & 0x7FF00000);
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const int m = warp_max_i(e[v]) >> 20;
+                if (lane == 0) {
+                    const int ec = m == 0 || m - 1022 < -1000 ? 0 : m - 1022;  // as exp_bound
+                    Ecol[c + v] = ec;
+                    st_cluster_s32(map_peer(smem_addr(&Ecol[c + v]), peer), ec);
+                }
+            }
         }
-        for (; r < r1; r += 32) e = max(e, exp_bound(g[r]));
-        e = warp_max_i(e);
-        if (lane == 0) {
-            e = e < -1000 ? 0 : e;
-            Ecol[c] = e;
-            st_cluster_s32(map_peer(smem_addr(&Ecol[c]), peer), e);
-        }
-    }
     if (tid == 0) {
         s_fail = 0;
         for (int b = 0; b < kGramBufs; ++b) {

@@ -139,6 +139,8 @@ def lib():
             L.hsvd_mlp_adam.argtypes = [_p, _p, _p, _p, _int, ctypes.c_float, ctypes.c_float, ctypes.c_float,
                                         ctypes.c_float, _p]
             L.hsvd_mlp_adam.restype = _int
+            L.hsvd_release_scratch.argtypes = []
+            L.hsvd_release_scratch.restype = _int
             L.hsvd_default_batch_opts.argtypes = [ctypes.POINTER(HsvdBatchOpts)]
             L.hsvd_default_batch_opts.restype = None
             L.hsvd_solve_batched.argtypes = [_i64, _p, _p, _p, _p, _p, _dbl, _int, _p, _p, _p, _p, _p, _p]
@@ -148,6 +150,14 @@ def lib():
             L.hsvd_solve_batched_ex.restype = _int
             _lib = L
     return _lib
+
+
+def hsvd_release_scratch():
+    """Give the device scratch that the library keeps between calls (at most
+    256 MB per device) back to the current device."""
+    st = lib().hsvd_release_scratch()
+    if st != HSVD_OK:
+        raise HsvdError(st)
 
 
 def hsvd_status_string(status):

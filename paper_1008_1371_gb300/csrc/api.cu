@@ -364,12 +364,19 @@ int solve_blocked_core(const double *G, int64_t m, int64_t n, int64_t ldg, const
     // stream orders the reuse of the slot's buffers kRing steps later.  The
     // group size keeps the graph near kMaxNodes kernel nodes per sweep: the
     // GPU dispatches graph nodes at a bounded rate (about 2 us per node
-    // measured), which would otherwise bound the sweep.  From n = 4096 a
-    // visit's kernels take hundreds of microseconds and twice the nodes
-    // (smaller groups, more overlap) measured faster (Haar 4096, split
-    // precision: 1263 against 1275 ms; 11 visits per group: 1344 ms).
+    // measured), which would otherwise bound the sweep.  From n = 2048 a
+    // visit's kernels take long enough for twice the nodes, smaller groups and
+    // more overlap (split precision: n = 2048 265 -> 261 ms; Haar 4096 1230 ms
+    // with a quarter of them, 1160 so, 1172 with twice as many).  Where a visit's
+    // kernels are as short as their dispatch and a step's fill the chip, all of a
+    // step goes into one group, and the capture costs a tenth (b = 16: n = 160
+    // 7.9 -> 7.5 ms, 256 12.5 -> 11.1, 301 16.8 -> 15.1, 400 26.0 -> 24.5); up to
+    // n = 511 half the nodes are better (450: 32.8 -> 31.2, 500: 35.6 -> 33.5).
     const int kpv = prec ? 4 : 3;  // kernels per visit
-    const int64_t max_nodes = n_pad >= 4096 ? 2 * kMaxNodes : kMaxNodes;
+    const int64_t max_nodes = n_pad >= 2048                ? 2 * kMaxNodes
+                              : b == 16 && n_pad <= 416    ? 1
+                              : n_pad < 512                ? kMaxNodes / 2
+                                                           : kMaxNodes;
     const int grp = (int)std::min<int64_t>(npairs, std::max<int64_t>(1, ((int64_t)nb * npairs * kpv + max_nodes - 1) /
                                                                           max_nodes));
     auto capture_pairs = [&](const int *tab, const int *vis, const std::vector<int> &nact,

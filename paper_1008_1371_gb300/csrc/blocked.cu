@@ -117,25 +117,26 @@ k_gram(const double *__restrict__ G, int64_t rows, int64_t ldg, int parts, int i
     const int xw = ((tid >> 5) + 8 - (item + item / 152) % 8) % 8;
     const int ec = ((tid & 31) + 32 * xw) % B;  // its column (all of B = 16 twice)
     auto rows_of = [&](auto extra) {
-        slices([&]() {
 #pragma unroll 4
-            for (int r = 0; r < kGramKS; ++r) {
-                int f = 0;
+        for (int r = 0; r < kGramKS; ++r) {
+            int f = 0;
 #pragma unroll
-                for (int i = 0; i < TM; ++i)
+            for (int i = 0; i < TM; ++i)
 #pragma unroll
-                    for (int j = i + 1; j < TM; ++j, ++f) {
-                        fx[f] = fma(Xs[r][tx + 16 * i], Xs[r][ty + 16 * j], fx[f]);
-                        fy[f] = fma(Ys[r][tx + 16 * i], Ys[r][ty + 16 * j], fy[f]);
-                    }
+                for (int j = i + 1; j < TM; ++j, ++f) {
+                    fx[f] = fma(Xs[r][tx + 16 * i], Xs[r][ty + 16 * j], fx[f]);
+                    fy[f] = fma(Ys[r][tx + 16 * i], Ys[r][ty + 16 * j], fy[f]);
+                }
 #pragma unroll
-                for (int i = 0; i < TM; ++i) dg[i] = fma(P[r][tx + 16 * i], P[r][ty + 16 * i], dg[i]);
-                if constexpr (decltype(extra)::value) ex = fma(Ys[r][ec], Ys[r][ec], ex);
-            }
-        });
+            for (int i = 0; i < TM; ++i) dg[i] = fma(P[r][tx + 16 * i], P[r][ty + 16 * i], dg[i]);
+            if constexpr (decltype(extra)::value) ex = fma(Ys[r][ec], Ys[r][ec], ex);
+        }
     };
-    if (xw < kExtra) rows_of(std::true_type{});
-    else rows_of(std::false_type{});
+    // the warps part inside a slice only: its barriers are the whole CTA's
+    slices([&]() {
+        if (xw < kExtra) rows_of(std::true_type{});
+        else rows_of(std::false_type{});
+    });
     double *ox = out, *oy = out + 2 * bs;
     int f = 0;
 #pragma unroll

@@ -208,48 +208,60 @@ cudaError_t cluster_config(int count, int C, const ClShape &s, cudaStream_t st, 
     return e;
 }
 
-// Cluster size for a batch too short for the SMs, 0: the queue of groups.  Both
-// are estimated in cycles of a sweep from the FP64 instructions a warp issues
-// (64 cycles on its quarter of an SM, 16 on a whole one): on groups the
-// longest factor has an SM to itself or the SMs share the work evenly; on
-// clusters the longest factor or the work over the clusters resident at once.
-// Clusters must be estimated a fifth faster: their warps form each rotation
-// for one pair only, so they win by spreading, not by work.  Measured (n
-// uniform on [16, 256]): see widen_for_tail.
-int few_clusters(const std::vector<BTask> &tasks, int sms) {
+// Cluster size for a batch of at most one factor per SM, 0: the queue of groups.
+// Both are estimated in cycles a step, times the steps of a sweep, from the FP64
+// instructions a warp issues (64 cycles on its quarter of an SM) and what a step
+// takes besides them, fitted to whole calls on n = 4 to 256: on groups a factor
+// has an SM to itself, at most a warp per pair forms dots, and the packed
+// rotations and three barriers take 10,200 cycles; on clusters a warp per pair
+// has a rotation of its own (56 instructions) and one barrier, 2,000.  0.8: the
+// later sweeps skip rotations and kept dots.  The clusters share the SMs' FP64
+// pipes, which no residency count shows (114 factors of n = 40: 3,200 cycles by
+// the longest factor, 17,000 by the pipes), at 250 cycles a CTA.  Clusters must be
+// estimated a fifth faster than groups; a smaller cluster must win 6 % (fewer
+// and fuller CTAs spread less evenly).  Measured, whole calls in ms, groups / this
+// choice: n = 8: 4 factors 0.53 / 0.40, 152 2.13 / 2.00; n = 16: 4 1.00 / 0.64, 152
+// 2.71 / 2.49; n = 40: 38 3.9 / 3.2, 114 4.6 / 4.6 (clusters of 16: 8.6); n = 64:
+// 38 7.2 / 4.5, 76 7.9 / 7.9 (8.5); n = 256: 38 220 / 150; 1024 x 8: 4 1.17 / 0.77.
+int few_clusters(const std::vector<BTask> &tasks, int sms, cudaStream_t st) {
     if ((int)tasks.size() > sms) return 0;
-    double g_max = 0.0, g_sum = 0.0;
+    double groups = 0.0, pipes = 0.0, steps = 0.0;
+    int most = 0;  // pairs of the largest factor
     for (const BTask &t : tasks) {
         const double m = pw_rows_pad(t.m, t.n), n = t.n + (t.n & 1), half = n / 2;
-        const double work = half * (7.0 * m + 4.0 * n) / 32.0 * 16.0;
-        g_max = std::max(g_max, n * (work + 50.0 * 64.0 + 1000.0));
-        g_sum += n * (1.1 * work + 50.0 * 16.0 * ceil(half / 32.0));
+        const double rows = 0.8 * (7.0 * m + 4.0 * n) / 32.0;
+        groups = std::max(groups, n * (std::max(half, 4.0) * rows * 16.0 + 10200.0));
+        pipes += n * half * (rows + 56.0) * 16.0;
+        steps += n;
+        most = std::max(most, (t.n + 1) / 2);
     }
-    const double groups = std::max(g_max, g_sum / sms);
-    double best = 0.8 * groups;
+    const double line = 0.8 * groups;
+    double best = 0.0;
     int best_c = 0;
-    for (int C : {16, 8, 4}) {
+    for (int C : {16, 8, 4, 2, 1}) {
         const ClShape s = cluster_shape(tasks, C);
-        if (s.P > kMaxClPairs || s.smem > kClSmemMax) continue;
+        if (C > most || s.P > kMaxClPairs || s.smem > kClSmemMax) continue;
         double c_max = 0.0, c_sum = 0.0;
         for (const BTask &t : tasks) {
             const double m = pw_rows_pad(t.m, t.n), n = t.n + (t.n & 1);
             const double turns = ceil(ceil(n / 2 / C) / 4.0);  // pairs per quarter of an SM
-            const double c = n * (turns * (7.0 * m / 32.0 + 4.0 * n / 32.0 + 56.0) * 64.0 + 1200.0);
+            const double c = n * (turns * (0.8 * (7.0 * m + 4.0 * n) / 32.0 + 56.0) * 64.0 + 2000.0);
             c_max = std::max(c_max, c);
             c_sum += c;
         }
-        if (c_max > best) continue;
+        const double bound = best_c ? std::min(line, 0.94 * best) : line;
+        double c = std::max(c_max, (pipes + 250.0 * C * steps) / sms);
+        if (c >= bound) continue;
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[1];
         int resident = 0;
-        if (cluster_config((int)tasks.size(), C, s, nullptr, cfg, attr) != cudaSuccess ||
+        if (cluster_config((int)tasks.size(), C, s, st, cfg, attr) != cudaSuccess ||
             cudaOccupancyMaxActiveClusters(&resident, k_batched_cl, &cfg) != cudaSuccess || resident < 1) {
             cudaGetLastError();
             continue;
         }
-        const double c = std::max(c_max, c_sum / resident);
-        if (c < best) {
+        c = std::max(c, c_sum / resident);
+        if (c < bound) {
             best = c;
             best_c = C;
         }
@@ -569,7 +581,7 @@ int hsvd_solve_batched_ex(int64_t count, const double *const *G, const int64_t *
     std::vector<int> width(kBuckets, o.group_width ? o.group_width : cta);
     float ms_tune = 0.f;
     int tuned = 0;
-    const int C = (o.group_width || o.cta_threads) ? 0 : few_clusters(tasks, sms);
+    const int C = (o.group_width || o.cta_threads) ? 0 : few_clusters(tasks, sms, st);
     if (rc == HSVD_OK && o.group_width == 0 && C == 0) {
         std::vector<int> w;
         const bool cached = [&] {

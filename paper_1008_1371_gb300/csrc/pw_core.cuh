@@ -272,7 +272,7 @@ __device__ __forceinline__ int pw_finish_column(const double *g, const double *w
 // formed only when V is asked for.
 //
 // A step has three phases with a group barrier after each: the dots of every
-// pair by its warp (four pairs at a time), the rotations one pair per lane,
+// pair by its warp (up to four pairs at a time), the rotations one pair per lane,
 // and the column updates.  The rotation's chain of about 50 FP64 instructions
 // costs a warp the same for 1 or 32 pairs (64 cycles of its quarter of the
 // SM's FP64 pipe per instruction), so the pairs are packed into as few warps
@@ -350,11 +350,17 @@ __device__ void pw_solve(const double *__restrict__ G, int64_t ldg, int m, int n
     int sweep = 0, status = HSVD_NOT_CONVERGED, rule = HSVD_STOP_NONE;
     const int half = n_pad / 2;
     const int pwarp = (warp - first) & (kW - 1);  // which 32 pairs this warp rotates
+    // Pairs whose dots a warp forms together: four save half of the lanes' sums
+    // while every warp has some, else a pair's rows are the longer chain (110
+    // factors of 2048 x 16: 5.9 ms with four on 2 of the 8 warps, 3.5 ms with one on
+    // each; 608 of n = 8: 0.46 and 0.39; of n = 32: 3.37 with four on 4, 3.56 with
+    // two on 8).
+    const int per = min(4, (half + kW - 1) / kW);
     for (sweep = 1; sweep <= max_sweeps; ++sweep) {
         for (int s = 0; s < n_pad; ++s) {
-            // the dots, four pairs at a time, reduced together
-            for (int k0 = 4 * warp; k0 < half; k0 += 4 * kW) {
-                const int nb = min(4, half - k0);
+            // the dots, `per` pairs at a time, reduced together
+            for (int k0 = per * warp; k0 < half; k0 += per * kW) {
+                const int nb = min(per, half - k0);
                 int my_p = 0, my_q = 0, my_need = 0;
                 if (lane < nb) {
                     int a, b;

@@ -202,7 +202,7 @@ cudaError_t cluster_config(int count, int C, const ClShape &s, cudaStream_t st, 
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaFuncSetAttribute(k_batched_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
+    cudaError_t e = cudaFuncSetAttribute(k_batched_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemMax);
     if (e == cudaSuccess && C > 8)
         e = cudaFuncSetAttribute(k_batched_cl, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;

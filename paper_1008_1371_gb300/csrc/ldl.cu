@@ -775,6 +775,9 @@ k_ldl_persist(const double *__restrict__ M, int64_t ldm, double *__restrict__ W,
 
 constexpr int kUpdGrid = 608;
 
+// dynamic shared memory of k_ldl_persist: two pivot columns and two tables
+constexpr size_t persist_smem(int64_t n) { return (size_t)n * (2 * sizeof(double) + 2 * sizeof(int)); }
+
 }  // namespace
 
 // M (n x n, ldm, device, symmetric; read-only) -> G (n x n, ldg, device) and
@@ -820,9 +823,11 @@ int ldl_factor(const double *M, int64_t n, int64_t ldm, double *G, int64_t ldg, 
         ok(cudaMemset2DAsync(G, sizeof(double) * ldg, 0, sizeof(double) * n, n, st));
         ok(cudaMemsetAsync(bsize, 1, (size_t)n, st));
         if (persist) {
-            const size_t smem = (size_t)n * (2 * sizeof(double) + 2 * sizeof(int));
+            const size_t smem = persist_smem(n);
             ok(cudaMemsetAsync(slots, 0, sizeof(LdlSlot) * nslots, st));
-            ok(cudaFuncSetAttribute(k_ldl_persist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            // the limit for every n: it belongs to the function, not to this launch
+            ok(cudaFuncSetAttribute(k_ldl_persist, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)persist_smem(kPersistMaxN)));
             int n_int = (int)n;
             void *args[] = {(void *)&M, &ldm, &W, &n_int, &G, &ldg, &perm, &Dblk, &bsize, &state, &slots};
             ok(cudaLaunchCooperativeKernel((const void *)k_ldl_persist, dim3(grid), dim3(kPT), args, smem, st));

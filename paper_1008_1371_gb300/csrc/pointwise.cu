@@ -9,6 +9,8 @@ namespace hsvd {
 namespace {
 
 constexpr int kThreads = 1024;
+// of k_pointwise: G and 20 bytes a column within 200 KB (pointwise_fits, so n <= 158), and 12 more a column
+constexpr size_t kOneCtaSmemMax = 200 * 1024 + 158 * 12;
 
 __global__ void __launch_bounds__(kThreads, 1)
 k_pointwise(const double *__restrict__ G, int64_t ldg, int m, int n, const int8_t *__restrict__ J,
@@ -61,7 +63,8 @@ cudaError_t launch_pointwise(const double *G, int64_t ldg, int m, int n, const i
         const size_t smem = pw_cluster_smem(m_pad, n_pad, P, V != nullptr);
         if (C / 2 >= half && C > 1) break;
         if (smem > kClSmemMax || P > kMaxClPairs || (P > 4 && C < kMaxCl)) continue;
-        cudaError_t e = cudaFuncSetAttribute(k_pointwise_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e =
+            cudaFuncSetAttribute(k_pointwise_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemMax);
         if (e == cudaSuccess && C > 8)
             e = cudaFuncSetAttribute(k_pointwise_cl, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
@@ -89,8 +92,8 @@ cudaError_t launch_pointwise(const double *G, int64_t ldg, int m, int n, const i
                                   sigma, U, ldu, V, ldv, dev_out, dev_rot);
     }
     const size_t smem = (size_t)m_pad * n_pad * sizeof(double) + pw_aux_bytes(n_pad);
-    cudaError_t e = cudaFuncSetAttribute(k_pointwise, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e =
+        cudaFuncSetAttribute(k_pointwise, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOneCtaSmemMax);
     if (e != cudaSuccess) return e;
     k_pointwise<<<1, kThreads, smem, st>>>(G, ldg, m, n, J, m_pad, n_pad, tol, tstop, max_sweeps, sort, Wws,
                                            sigma, U, ldu, V, ldv, dev_out, dev_rot);

@@ -13,6 +13,9 @@ namespace cg = cooperative_groups;
 
 constexpr int kMaxCl = 16;       // CTAs of a cluster at most (16 is beyond the portable 8)
 constexpr int kMaxClPairs = 16;  // pairs (warps) per CTA at most
+// Dynamic shared memory of a CTA at most.  The kernels' limit is set to it, whatever
+// a call needs: the limit belongs to the function, so a call that lowered it to
+// its own size would fail another host thread's launch.
 constexpr size_t kClSmemMax = 220 * 1024;
 
 // dynamic shared memory of a CTA with P pairs

@@ -469,9 +469,11 @@ k_qr_update(double *__restrict__ C, int64_t ldc, int64_t m, int c0, int ncols, c
 template <bool SMEM>
 cudaError_t launch_panel_cl(double *A, int64_t lda, int64_t m, int j0, int w, int rp, double *tau, cudaStream_t st) {
     const size_t smem = SMEM ? (size_t)kQB * rp * sizeof(double) : 0;
+    // the limit for every rp: it belongs to the function, not to this launch
+    constexpr size_t kMax = SMEM ? (size_t)kQB * kPanelClMaxRows * sizeof(double) : 0;
     cudaError_t e = cudaFuncSetAttribute(k_qr_panel_cl<SMEM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_qr_panel_cl<SMEM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k_qr_panel_cl<SMEM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMax);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kPanelCl);

@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <functional>
 #include <type_traits>
 #include <vector>
 
@@ -806,7 +807,11 @@ int ldl_factor(const double *M, int64_t n, int64_t ldm, double *G, int64_t ldg, 
     const bool persist = n <= kPersistMaxN;
     const int grid = (int)std::min<int64_t>(sms, std::max<int64_t>(1, n / 6));
     const size_t nslots = persist ? 2 * (size_t)grid : 0;
-    if (!ok(scratch_alloc((void **)&W, sizeof(double) * n * (n + 2), st)) ||
+    const double *m_end = M + (n - 1) * ldm + n, *g_end = G + (n - 1) * ldg + n;
+    const bool overlap = persist && std::less<const double *>()(M, g_end) && std::less<const double *>()(G, m_end);
+    double *Mc = nullptr;
+    if ((overlap && !ok(scratch_alloc((void **)&Mc, sizeof(double) * n * n, st))) ||
+        !ok(scratch_alloc((void **)&W, sizeof(double) * n * (n + 2), st)) ||
         !ok(scratch_alloc((void **)&Dblk, sizeof(double) * 4 * n, st)) ||
         !ok(scratch_alloc((void **)&perm, sizeof(int) * n, st)) ||
         !ok(scratch_alloc((void **)&bsize, (size_t)n, st)) ||
@@ -820,9 +825,17 @@ int ldl_factor(const double *M, int64_t n, int64_t ldm, double *G, int64_t ldg, 
         s0.rank = (int)n;
         std::vector<int> p;
         ok(cudaMemcpyAsync(state, &s0, sizeof s0, cudaMemcpyHostToDevice, st));
-        ok(cudaMemset2DAsync(G, sizeof(double) * ldg, 0, sizeof(double) * n, n, st));
         ok(cudaMemsetAsync(bsize, 1, (size_t)n, st));
+        // L starts as zeros in G, which may lie in M's memory: M is copied first
+        auto zero_g = [&]() { ok(cudaMemset2DAsync(G, sizeof(double) * ldg, 0, sizeof(double) * n, n, st)); };
         if (persist) {
+            if (Mc) {
+                ok(cudaMemcpy2DAsync(Mc, sizeof(double) * n, M, sizeof(double) * ldm, sizeof(double) * n, n,
+                                     cudaMemcpyDeviceToDevice, st));
+                M = Mc;
+                ldm = n;
+            }
+            zero_g();
             const size_t smem = persist_smem(n);
             ok(cudaMemsetAsync(slots, 0, sizeof(LdlSlot) * nslots, st));
             // the limit for every n: it belongs to the function, not to this launch
@@ -836,6 +849,7 @@ int ldl_factor(const double *M, int64_t n, int64_t ldm, double *G, int64_t ldg, 
             for (int64_t i = 0; i < n; ++i) p[(size_t)i] = (int)i;
             ok(cudaMemcpy2DAsync(W, sizeof(double) * n, M, sizeof(double) * ldm, sizeof(double) * n, n,
                                  cudaMemcpyDeviceToDevice, st));
+            zero_g();
             ok(cudaMemcpyAsync(perm, p.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
             k_ldl_max0<<<kUpdGrid, kUpdThreads, 0, st>>>(W, n, (int)n, mx, state);
             ok(cudaGetLastError());
@@ -857,6 +871,7 @@ int ldl_factor(const double *M, int64_t n, int64_t ldm, double *G, int64_t ldg, 
         if (rank) *rank = fin.rank;
         if (launches) *launches += persist ? 2 : 2 + 3 * n;
     }
+    if (Mc) cudaFreeAsync(Mc, st);
     if (W) cudaFreeAsync(W, st);
     if (Dblk) cudaFreeAsync(Dblk, st);
     if (perm) cudaFreeAsync(perm, st);

@@ -223,7 +223,8 @@ cudaError_t cluster_config(int count, int C, const ClShape &s, cudaStream_t st, 
 // choice: n = 8: 4 factors 0.53 / 0.40, 152 2.13 / 2.00; n = 16: 4 1.00 / 0.64, 152
 // 2.71 / 2.49; n = 40: 38 3.9 / 3.2, 114 4.6 / 4.6 (clusters of 16: 8.6); n = 64:
 // 38 7.2 / 4.5, 76 7.9 / 7.9 (8.5); n = 256: 38 220 / 150; 1024 x 8: 4 1.17 / 0.77.
-int few_clusters(const std::vector<BTask> &tasks, int sms, cudaStream_t st) {
+int few_clusters(const std::vector<BTask> &tasks, const StreamLimits &limits, cudaStream_t st) {
+    const int sms = limits.sms;
     if ((int)tasks.size() > sms) return 0;
     double groups = 0.0, pipes = 0.0, steps = 0.0;
     int most = 0;  // pairs of the largest factor
@@ -240,7 +241,7 @@ int few_clusters(const std::vector<BTask> &tasks, int sms, cudaStream_t st) {
     int best_c = 0;
     for (int C : {16, 8, 4, 2, 1}) {
         const ClShape s = cluster_shape(tasks, C);
-        if (C > most || s.P > kMaxClPairs || s.smem > kClSmemMax) continue;
+        if (C > most || C > limits.cluster || s.P > kMaxClPairs || s.smem > kClSmemMax) continue;
         double c_max = 0.0, c_sum = 0.0;
         for (const BTask &t : tasks) {
             const double m = pw_rows_pad(t.m, t.n), n = t.n + (t.n & 1);
@@ -581,7 +582,7 @@ int hsvd_solve_batched_ex(int64_t count, const double *const *G, const int64_t *
     std::vector<int> width(kBuckets, o.group_width ? o.group_width : cta);
     float ms_tune = 0.f;
     int tuned = 0;
-    const int C = (o.group_width || o.cta_threads) ? 0 : few_clusters(tasks, sms, st);
+    const int C = (o.group_width || o.cta_threads) ? 0 : few_clusters(tasks, stream_limits(st), st);
     if (rc == HSVD_OK && o.group_width == 0 && C == 0) {
         std::vector<int> w;
         const bool cached = [&] {

@@ -399,6 +399,13 @@ cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st);
 // identity of the current context, 0 if it cannot be read
 unsigned long long current_context_id();
 
+// limits.cu: SMs that a launch on the stream may use at once, and the CTAs of a
+// cluster that they are sure to hold
+struct StreamLimits {
+    int sms, cluster;
+};
+StreamLimits stream_limits(cudaStream_t st);
+
 // hypqr.cu: the hyperbolic QR of G^T for a wide G (m < n).  Device buffers,
 // filled by the caller: A, Vr (n x m), C (m x m), z (n), beta (m), cperm,
 // rswap (m), s (n), bsize (m), state and mx (hypqr_state_bytes,

@@ -799,13 +799,10 @@ int ldl_factor(const double *M, int64_t n, int64_t ldm, double *G, int64_t ldg, 
         if (e != cudaSuccess && rc == HSVD_OK) rc = HSVD_ERR_CUDA;
         return e == cudaSuccess;
     };
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // one launch while the pivot columns fit shared memory: a CTA for every six
-    // columns, at most one per SM
-    const bool persist = n <= kPersistMaxN;
-    const int grid = (int)std::min<int64_t>(sms, std::max<int64_t>(1, n / 6));
+    // columns, at most one per SM that the stream may use
+    bool persist = n <= kPersistMaxN;
+    const int grid = (int)std::min<int64_t>(stream_limits(st).sms, std::max<int64_t>(1, n / 6));
     const size_t nslots = persist ? 2 * (size_t)grid : 0;
     const double *m_end = M + (n - 1) * ldm + n, *g_end = G + (n - 1) * ldg + n;
     const bool overlap = persist && std::less<const double *>()(M, g_end) && std::less<const double *>()(G, m_end);
@@ -843,8 +840,16 @@ int ldl_factor(const double *M, int64_t n, int64_t ldm, double *G, int64_t ldg, 
                                     (int)persist_smem(kPersistMaxN)));
             int n_int = (int)n;
             void *args[] = {(void *)&M, &ldm, &W, &n_int, &G, &ldg, &perm, &Dblk, &bsize, &state, &slots};
-            ok(cudaLaunchCooperativeKernel((const void *)k_ldl_persist, dim3(grid), dim3(kPT), args, smem, st));
-        } else {
+            const cudaError_t e =
+                cudaLaunchCooperativeKernel((const void *)k_ldl_persist, dim3(grid), dim3(kPT), args, smem, st);
+            if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+                cudaGetLastError();  // refused: the three kernels need no CTAs at the same time
+                persist = false;
+            } else {
+                ok(e);
+            }
+        }
+        if (!persist) {
             p.resize((size_t)n);
             for (int64_t i = 0; i < n; ++i) p[(size_t)i] = (int)i;
             ok(cudaMemcpy2DAsync(W, sizeof(double) * n, M, sizeof(double) * ldm, sizeof(double) * n, n,

@@ -3,6 +3,8 @@
 // warp per pair of a step (pw_cluster.cuh), and for the shapes whose columns do not fit its
 // shared memory (two columns of more than about 6,900 rows) k_pointwise, one
 // CTA running pw_solve (pw_core.cuh) with G in shared memory and W in global.
+#include <algorithm>
+
 #include "pw_cluster.cuh"
 
 namespace hsvd {
@@ -58,11 +60,13 @@ cudaError_t launch_pointwise(const double *G, int64_t ldg, int m, int n, const i
     const int m_pad = pw_rows_pad(m, n);
     const int half = n_pad / 2;
     // the smallest cluster with at most four pairs a CTA, else the largest
-    for (int C = 1; C <= kMaxCl; C *= 2) {
+    int max_c = 1;  // of the clusters that the stream's SMs hold
+    for (const int limit = stream_limits(st).cluster; 2 * max_c <= std::min(kMaxCl, limit);) max_c *= 2;
+    for (int C = 1; C <= max_c; C *= 2) {
         const int P = (half + C - 1) / C;
         const size_t smem = pw_cluster_smem(m_pad, n_pad, P, V != nullptr);
         if (C / 2 >= half && C > 1) break;
-        if (smem > kClSmemMax || P > kMaxClPairs || (P > 4 && C < kMaxCl)) continue;
+        if (smem > kClSmemMax || P > kMaxClPairs || (P > 4 && C < max_c)) continue;
         cudaError_t e =
             cudaFuncSetAttribute(k_pointwise_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemMax);
         if (e == cudaSuccess && C > 8)

@@ -470,8 +470,9 @@ int hsvd_mlp_adam(float *params, float *m, float *v, const float *grad, int t, f
 
 /*
  * The calls take their device scratch from a pool of the library's own, which
- * keeps at most 256 MB per device between calls.  hsvd_release_scratch gives
- * what no call is using back to the device (the current device).
+ * keeps at most 256 MB per device (and context, where a program has several)
+ * between calls.  hsvd_release_scratch gives what no call is using back to the
+ * current device (from the current context's pool).
  */
 int hsvd_release_scratch(void);
 

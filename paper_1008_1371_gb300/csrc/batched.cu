@@ -5,13 +5,14 @@
 // Work distribution.  The host sorts the factors by (group width, n), both
 // decreasing, and the kernel's CTAs (1024 threads, or 512 with twice the
 // registers a thread, one per SM, launched once and captured in a CUDA graph)
-// take them from one atomic counter: the largest
-// first, so the long factors start early and the short ones fill the tail.
+// take them in that order from one atomic counter (EVEN: but for every group's
+// first): the largest first, so the long factors start early and the short ones
+// fill the tail.
 // A CTA starts as one group of 1024 threads.  When the next factor in the
 // queue asks for a narrower group, the CTA splits into two groups of 512
 // (each with half the shared memory and its own named barrier), and a 512
 // group splits again into two groups of 256; every group then takes factors
-// from the same counter on its own.  The queue order makes the widths
+// from the counter on its own.  The queue order makes the widths
 // non-increasing, so a group never has to grow back.
 //
 // Residency.  In its group's shared memory a factor keeps G and W when both
@@ -49,7 +50,9 @@ struct BTask {
 struct BArgs {
     const BTask *tasks;
     int count;
-    int *counter;
+    int *counter;        // factors taken (EVEN: beyond the first ones)
+    int width;           // EVEN: the width of every factor
+    int firsts;          // EVEN: factors given out at the start, one a group
     int max_sweeps, sort;
     double tstop;        // tangent threshold of the early stop, 0 = off
     double *ws;          // grid x ws_stride doubles
@@ -61,7 +64,7 @@ struct BArgs {
 
 __device__ __forceinline__ int bar_id(int width, int g) { return width == 1024 ? 0 : (width == 512 ? 1 + g : 3 + g); }
 
-template <int NT>
+template <int NT, bool FEW>
 __device__ void solve_task(const BArgs &A, int k, int g, unsigned char *sm, size_t budget, double *wsg,
                            PwScalars *sc) {
     const BTask t = A.tasks[k];
@@ -87,48 +90,60 @@ __device__ void solve_task(const BArgs &A, int k, int g, unsigned char *sm, size
     const int where = a.gs < n_pad ? 2 : (a.ws < n_pad ? 1 : 0);
     const int bar = bar_id(NT, g);
     int *res = A.res + 3 * (size_t)t.idx;
-    pw_solve<NT>(t.G, t.ldg, t.m, t.n, t.J, m_pad, n_pad, t.tol, A.tstop, A.max_sweeps, A.sort, a, sc[bar], t.sigma,
+    pw_solve<NT, FEW>(t.G, t.ldg, t.m, t.n, t.J, m_pad, n_pad, t.tol, A.tstop, A.max_sweeps, A.sort, a, sc[bar], t.sigma,
                  t.U, t.ldu, t.V, t.ldv, &res[0], &res[1], &A.rot[t.idx], &res[2], bar, NT == 512 ? 2 * g : g);
     if ((threadIdx.x & (NT - 1)) == 0) A.where[t.idx] = where;
 }
 
+// EVEN is for queues of one width narrower than a CTA: the first factor of every
+// group f is dealt out, back and forth, so that no SM has three while another has
+// one.  By the counter the CTAs that start first can take one for each of their
+// groups: 200 factors of n = 64 then take 9.6 or 12.7 ms from process to process, 304
+// of n = 256 on 256 threads 613 or 704; dealt out 9.6 and 450.  It is a template
+// argument for the registers of the other kernels (1 % there).
+__device__ __forceinline__ int first_factor(int f) {
+    return f * (int)gridDim.x + ((f & 1) ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x);
+}
+
 // Group g of width NT: solves factors from the queue, starting with factor k
 // (k < 0: take one from the counter first).
-template <int NT>
+template <int NT, bool FEW, bool EVEN, int CTA>
 __device__ void group_loop(const BArgs &A, int k, int g, unsigned char *sm, size_t budget, double *wsg,
                            int64_t wsg_len, PwScalars *sc, int *fetch) {
     const int bar = bar_id(NT, g);
     const int tid = threadIdx.x & (NT - 1);
     for (;;) {
         if (k < 0) {
-            if (tid == 0) fetch[bar] = atomicAdd(A.counter, 1);
+            if (tid == 0) fetch[bar] = (EVEN ? A.firsts : 0) + atomicAdd(A.counter, 1);
             grp_sync<NT>(bar);
             k = fetch[bar];
             grp_sync<NT>(bar);
         }
         if (k >= A.count) return;
-        if constexpr (NT > 256) {
-            if (A.tasks[k].width < NT) {
+        // small factors are all of one size bucket, so of one width: EVEN, or the CTA's
+        if constexpr (NT > 256 && !(FEW && !EVEN && CTA == 1024)) {
+            if ((EVEN ? A.width : A.tasks[k].width) < NT) {
                 const int sub = tid / (NT / 2);
-                group_loop<NT / 2>(A, sub == 0 ? k : -1, 2 * g + sub, sm + sub * (budget / 2), budget / 2,
-                                   wsg + sub * (wsg_len / 2), wsg_len / 2, sc, fetch);
+                const int other = EVEN ? first_factor((2 * g + 1) * (NT / 2) / A.width) : -1;
+                group_loop<NT / 2, FEW, EVEN, CTA>(A, sub == 0 ? k : other, 2 * g + sub, sm + sub * (budget / 2),
+                                                   budget / 2, wsg + sub * (wsg_len / 2), wsg_len / 2, sc, fetch);
                 return;
             }
         }
-        solve_task<NT>(A, k, g, sm, budget, wsg, sc);
+        if constexpr (!EVEN || NT < 1024) solve_task<NT, FEW>(A, k, g, sm, budget, wsg, sc);
         k = -1;
     }
 }
 
 // CTA threads: 1024 (64 registers a thread) or 512 (128: the per-thread
 // state of pw_solve without spills)
-template <int CTA>
+template <int CTA, bool FEW, bool EVEN>
 __global__ void __launch_bounds__(CTA, 1) k_batched(BArgs A, int smem_budget) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ PwScalars sc[kBarriers];
     __shared__ int fetch[kBarriers];
-    group_loop<CTA>(A, -1, 0, smem, (size_t)smem_budget, A.ws + (size_t)blockIdx.x * A.ws_stride, A.ws_stride, sc,
-                    fetch);
+    group_loop<CTA, FEW, EVEN, CTA>(A, EVEN ? first_factor(0) : -1, 0, smem, (size_t)smem_budget,
+                                    A.ws + (size_t)blockIdx.x * A.ws_stride, A.ws_stride, sc, fetch);
 }
 
 // A few factors, too few to fill the SMs one each: one cluster per factor, in
@@ -168,11 +183,6 @@ int64_t ws_stride_for(const std::vector<BTask> &tasks, int cta) {
         s = std::max(s, (need_bytes(t.m, t.n) + pw_aux_bytes(t.n + (t.n & 1))) * (size_t)(cta / t.width));
     return (int64_t)((s / sizeof(double) + 31) / 32 * 32);
 }
-
-struct Launch {
-    int grid = 0;
-    cudaError_t err = cudaSuccess;
-};
 
 // pairs a CTA and shared memory of the largest factor on clusters of C CTAs
 struct ClShape {
@@ -270,6 +280,12 @@ int few_clusters(const std::vector<BTask> &tasks, const StreamLimits &limits, cu
     return best_c;
 }
 
+void (*batched_kernel(int cta, bool few, bool even))(BArgs, int) {
+    if (cta == 512) return few ? k_batched<512, true, false> : k_batched<512, false, false>;
+    return few ? (even ? k_batched<1024, true, true> : k_batched<1024, true, false>)
+               : (even ? k_batched<1024, false, true> : k_batched<1024, false, false>);
+}
+
 // Runs the persistent kernel over `tasks` (already in queue order), or with
 // C > 0 one cluster of C CTAs per factor, as one captured graph: counter reset
 // + the launch.
@@ -277,7 +293,11 @@ cudaError_t run_batch(const std::vector<BTask> &tasks, int max_sweeps, int sort,
                       int grid, int cta, int C, int *res, long long *rot, int *where, cudaStream_t st, float *ms) {
     const int count = (int)tasks.size();
     const int64_t stride = C ? 0 : ws_stride_for(tasks, cta);
-    void (*kern)(BArgs, int) = cta == 512 ? k_batched<512> : k_batched<1024>;
+    bool few = true;  // every factor has few pairs (pw_solve)
+    for (const BTask &t : tasks) few = few && t.n <= kPwFew;
+    bool even = cta == 1024 && tasks[0].width < cta;  // one width, narrower than a CTA
+    for (const BTask &t : tasks) even = even && t.width == tasks[0].width;
+    void (*kern)(BArgs, int) = batched_kernel(cta, few, even);
     const ClShape shape = C ? cluster_shape(tasks, C) : ClShape{};
     auto launch = [&](const BArgs &A, cudaStream_t on) -> cudaError_t {
         if (C) {
@@ -302,6 +322,8 @@ cudaError_t run_batch(const std::vector<BTask> &tasks, int max_sweeps, int sort,
     A.tasks = d_tasks;
     A.count = count;
     A.counter = d_counter;
+    A.width = tasks[0].width;
+    A.firsts = grid * (cta / A.width);
     A.max_sweeps = max_sweeps;
     A.sort = sort;
     A.tstop = tstop;

@@ -14,6 +14,7 @@ constexpr int kThreads = 1024;
 // of k_pointwise: G and 20 bytes a column within 200 KB (pointwise_fits, so n <= 158), and 12 more a column
 constexpr size_t kOneCtaSmemMax = 200 * 1024 + 158 * 12;
 
+template <bool FEW>
 __global__ void __launch_bounds__(kThreads, 1)
 k_pointwise(const double *__restrict__ G, int64_t ldg, int m, int n, const int8_t *__restrict__ J,
             int m_pad, int n_pad, double tol, double tstop, int max_sweeps, int sort, double *__restrict__ W,
@@ -26,7 +27,7 @@ k_pointwise(const double *__restrict__ G, int64_t ldg, int m, int n, const int8_
     sh.gs = n_pad;
     sh.Wg = W;
     pw_carve(sh, smem + (size_t)m_pad * n_pad, n_pad);
-    pw_solve<kThreads>(G, ldg, m, n, J, m_pad, n_pad, tol, tstop, max_sweeps, sort, sh, sc, sigma, U, ldu, V,
+    pw_solve<kThreads, FEW>(G, ldg, m, n, J, m_pad, n_pad, tol, tstop, max_sweeps, sort, sh, sc, sigma, U, ldu, V,
                        ldv, &out[0], &out[1], rot_out, &out[2], 0, 0);
 }
 
@@ -95,11 +96,12 @@ cudaError_t launch_pointwise(const double *G, int64_t ldg, int m, int n, const i
         return cudaLaunchKernelEx(&cfg, k_pointwise_cl, G, ldg, m, n, J, P, tol, tstop, max_sweeps, sort,
                                   sigma, U, ldu, V, ldv, dev_out, dev_rot);
     }
+    auto kern = n <= kPwFew ? k_pointwise<true> : k_pointwise<false>;
     const size_t smem = (size_t)m_pad * n_pad * sizeof(double) + pw_aux_bytes(n_pad);
     cudaError_t e =
-        cudaFuncSetAttribute(k_pointwise, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOneCtaSmemMax);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOneCtaSmemMax);
     if (e != cudaSuccess) return e;
-    k_pointwise<<<1, kThreads, smem, st>>>(G, ldg, m, n, J, m_pad, n_pad, tol, tstop, max_sweeps, sort, Wws,
+    kern<<<1, kThreads, smem, st>>>(G, ldg, m, n, J, m_pad, n_pad, tol, tstop, max_sweeps, sort, Wws,
                                            sigma, U, ldu, V, ldv, dev_out, dev_rot);
     return cudaGetLastError();
 }

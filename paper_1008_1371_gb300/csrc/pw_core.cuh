@@ -265,6 +265,90 @@ __device__ __forceinline__ int pw_finish_column(const double *g, const double *w
     return err;
 }
 
+// The dots of step s for the group's pairs, PER pairs of a warp at a time, reduced
+// together: a lane ends with one of the sums, z = a_pq of pair u in the lanes whose
+// `part` is PART_Z, and where a pair's kept dots are missing x = a_pp and y = a_qq in
+// two others.
+template <int NT, int PER>
+__device__ __forceinline__ void pw_step_dots(const PwArrays &sh, int m_pad, int n_pad, int s) {
+    constexpr int kW = NT / kWarp;
+    const int tid = threadIdx.x & (NT - 1), lane = tid & 31, warp = tid >> 5, half = n_pad / 2;
+    for (int k0 = PER * warp; k0 < half; k0 += PER * kW) {
+        const int nb = min(PER, half - k0);
+        int my_p = 0, my_q = 0, my_need = 0;
+        if (lane < nb) {
+            int a, b;
+            modulus_pair(n_pad, s, k0 + lane, a, b);
+            my_p = sh.pos[a];
+            my_q = sh.pos[b];
+            sh.pq[k0 + lane] = my_p | (my_q << 16);
+            my_need = (pw_missing(sh.d[my_p]) ? 1 : 0) | (pw_missing(sh.d[my_q]) ? 2 : 0);
+        }
+        const bool any = __any_sync(0xffffffffu, my_need);
+        double v[PER][3];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            v[u][0] = v[u][1] = v[u][2] = 0.0;
+            if (u < nb) {
+                const int p = __shfl_sync(0xffffffffu, my_p, u), q = __shfl_sync(0xffffffffu, my_q, u);
+                const int need = __shfl_sync(0xffffffffu, my_need, u);
+                pw_dots_sel(need & 1, need & 2, sh.g(p, m_pad), sh.g(q, m_pad), m_pad, lane, v[u][0], v[u][1],
+                            v[u][2]);
+            }
+        }
+        const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4, h2 = lane & 2;
+        constexpr int PART_X = 0, PART_Y = PER == 4 ? 4 : 8, PART_Z = PER == 4 ? 2 : (PER == 2 ? 4 : 16);
+        double z;
+        int u, part;
+        if constexpr (PER == 4) {  // lanes with bits 4, 3 = u hold pair u's sums from the second level on
+            z = pw_fold(pw_fold(v[0][2], v[2][2], 16, h16), pw_fold(v[1][2], v[3][2], 16, h16), 8, h8);
+            if (any) {
+                const double x = pw_fold(pw_fold(v[0][0], v[2][0], 16, h16), pw_fold(v[1][0], v[3][0], 16, h16),
+                                         8, h8);
+                const double y = pw_fold(pw_fold(v[0][1], v[2][1], 16, h16), pw_fold(v[1][1], v[3][1], 16, h16),
+                                         8, h8);
+                // bit 1 set: z, else bit 2 clear: x, set: y
+                z = pw_fold(pw_fold(x, y, 4, h4), pw_xor_add(z, 4), 2, h2);
+            } else {
+                z = pw_xor_add(pw_xor_add(z, 4), 2);
+            }
+            u = (lane >> 3) & 3;
+            part = lane & 7;
+        } else if constexpr (PER == 2) {  // bit 4 = u
+            z = pw_xor_add(pw_fold(v[0][2], v[1][2], 16, h16), 8);
+            if (any) {
+                const double x = pw_fold(v[0][0], v[1][0], 16, h16), y = pw_fold(v[0][1], v[1][1], 16, h16);
+                // bit 2 set: z, else bit 3 clear: x, set: y
+                z = pw_fold(pw_fold(x, y, 8, h8), z, 4, h4);
+            } else {
+                z = pw_xor_add(z, 4);
+            }
+            z = pw_xor_add(z, 2);
+            u = lane >> 4;
+            part = lane & 15;
+        } else {
+            z = v[0][2];
+            if (any) {  // bit 4 set: z, else bit 3 clear: x, set: y
+                const double x = pw_fold(v[0][0], z, 16, h16), y = pw_xor_add(v[0][1], 16);
+                z = pw_fold(x, h16 ? x : y, 8, h8);
+            } else {
+                z = pw_xor_add(pw_xor_add(z, 16), 8);
+            }
+            z = pw_xor_add(pw_xor_add(z, 4), 2);
+            u = 0;
+            part = lane;
+        }
+        z = pw_xor_add(z, 1);
+        const int p = __shfl_sync(0xffffffffu, my_p, u), q = __shfl_sync(0xffffffffu, my_q, u);
+        const int need = __shfl_sync(0xffffffffu, my_need, u);
+        if (u < nb) {
+            if (part == PART_Z) sh.apq[k0 + u] = z;
+            if (part == PART_X && (need & 1)) sh.d[p] = z;
+            if (part == PART_Y && (need & 2)) sh.d[q] = z;
+        }
+    }
+}
+
 // Solves one factor; every thread of the group calls it.  Writes status, sweeps,
 // the rotation count and the stop rule (HSVD_STOP_*) through out_status /
 // out_sweeps / out_rot / out_rule (thread 0; out_rule may be null).  tstop > 0
@@ -278,8 +362,17 @@ __device__ __forceinline__ int pw_finish_column(const double *g, const double *w
 // SM's FP64 pipe per instruction), so the pairs are packed into as few warps
 // as hold them, warp `first` on; groups of one SM start at different warps so
 // that they do not share a quarter.  Measured (600 factors, n in [16, 256]):
-// 457 ms with a rotation per warp and every dot formed anew, 277 ms so.
-template <int NT>
+// 457 ms with a rotation per warp and every dot formed anew, 275 ms so.
+//
+// FEW is for factors of at most kPwFew columns, whose pairs are too few to come four
+// to a warp: one or two a warp instead, on eight warps (two a quarter of the SM)
+// where there are that many.  With four, 110 factors of 2048 x 16 took 5.9 ms, 3.5
+// so (3.8 with every pair on a warp of its own from dots to update), 304 of n = 8
+// 0.41 and 0.29 (0.38), 600 of n = 24 2.08 and 1.95 ms (4.65).  It is a template
+// argument because either form costs the other's registers (1 % of a batch of
+// large factors).
+constexpr int kPwFew = 32;
+template <int NT, bool FEW>
 __device__ void pw_solve(const double *__restrict__ G, int64_t ldg, int m, int n, const int8_t *__restrict__ J,
                          int m_pad, int n_pad, double tol, double tstop, int max_sweeps, int sort,
                          const PwArrays &sh, PwScalars &sc, double *__restrict__ sigma, double *__restrict__ U,
@@ -350,60 +443,13 @@ __device__ void pw_solve(const double *__restrict__ G, int64_t ldg, int m, int n
     int sweep = 0, status = HSVD_NOT_CONVERGED, rule = HSVD_STOP_NONE;
     const int half = n_pad / 2;
     const int pwarp = (warp - first) & (kW - 1);  // which 32 pairs this warp rotates
-    // Pairs whose dots a warp forms together: four save half of the lanes' sums
-    // while every warp has some, else a pair's rows are the longer chain (110
-    // factors of 2048 x 16: 5.9 ms with four on 2 of the 8 warps, 3.5 ms with one on
-    // each; 608 of n = 8: 0.46 and 0.39; of n = 32: 3.37 with four on 4, 3.56 with
-    // two on 8).
-    const int per = min(4, (half + kW - 1) / kW);
     for (sweep = 1; sweep <= max_sweeps; ++sweep) {
         for (int s = 0; s < n_pad; ++s) {
-            // the dots, `per` pairs at a time, reduced together
-            for (int k0 = per * warp; k0 < half; k0 += per * kW) {
-                const int nb = min(per, half - k0);
-                int my_p = 0, my_q = 0, my_need = 0;
-                if (lane < nb) {
-                    int a, b;
-                    modulus_pair(n_pad, s, k0 + lane, a, b);
-                    my_p = sh.pos[a];
-                    my_q = sh.pos[b];
-                    sh.pq[k0 + lane] = my_p | (my_q << 16);
-                    my_need = (pw_missing(sh.d[my_p]) ? 1 : 0) | (pw_missing(sh.d[my_q]) ? 2 : 0);
-                }
-                const bool any = __any_sync(0xffffffffu, my_need);
-                double v[4][3];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    v[u][0] = v[u][1] = v[u][2] = 0.0;
-                    if (u < nb) {
-                        const int p = __shfl_sync(0xffffffffu, my_p, u), q = __shfl_sync(0xffffffffu, my_q, u);
-                        const int need = __shfl_sync(0xffffffffu, my_need, u);
-                        pw_dots_sel(need & 1, need & 2, sh.g(p, m_pad), sh.g(q, m_pad), m_pad, lane, v[u][0], v[u][1],
-                                    v[u][2]);
-                    }
-                }
-                const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4, h2 = lane & 2;
-                // lanes with bits 4, 3 = u hold pair u's sums from the second level on
-                double z = pw_fold(pw_fold(v[0][2], v[2][2], 16, h16), pw_fold(v[1][2], v[3][2], 16, h16), 8, h8);
-                if (any) {
-                    const double x = pw_fold(pw_fold(v[0][0], v[2][0], 16, h16), pw_fold(v[1][0], v[3][0], 16, h16),
-                                             8, h8);
-                    const double y = pw_fold(pw_fold(v[0][1], v[2][1], 16, h16), pw_fold(v[1][1], v[3][1], 16, h16),
-                                             8, h8);
-                    // bit 1 set: z, else bit 2 clear: x, set: y
-                    z = pw_fold(pw_fold(x, y, 4, h4), pw_xor_add(z, 4), 2, h2);
-                } else {
-                    z = pw_xor_add(pw_xor_add(z, 4), 2);
-                }
-                z = pw_xor_add(z, 1);
-                const int u = (lane >> 3) & 3, part = lane & 7;
-                const int p = __shfl_sync(0xffffffffu, my_p, u), q = __shfl_sync(0xffffffffu, my_q, u);
-                const int need = __shfl_sync(0xffffffffu, my_need, u);
-                if (u < nb) {
-                    if (part == 2) sh.apq[k0 + u] = z;
-                    if (part == 0 && (need & 1)) sh.d[p] = z;
-                    if (part == 4 && (need & 2)) sh.d[q] = z;
-                }
+            if constexpr (FEW) {
+                if (half <= 8) pw_step_dots<NT, 1>(sh, m_pad, n_pad, s);
+                else pw_step_dots<NT, 2>(sh, m_pad, n_pad, s);
+            } else {
+                pw_step_dots<NT, 4>(sh, m_pad, n_pad, s);
             }
             grp_sync<NT>(bar);
             // the rotations, one pair per lane

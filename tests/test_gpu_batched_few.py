@@ -56,3 +56,14 @@ def test_dots_split_over_the_warps(api, m, n):
         b = api.hsvd_solve_batched([G], [J], api.make_batch_opts(group_width=w))
         assert b.sweeps[0] == one.sweeps and b.info.rotations == one.rotations
         assert torch.equal(b.sigma[0], one.sigma) and torch.equal(b.U[0], one.U) and torch.equal(b.V[0], one.V)
+
+
+@pytest.mark.parametrize("n,count", [(8, 160), (8, 700), (24, 305), (33, 700), (64, 161), (64, 460)])
+def test_queue_dealt_out(api, n, count):
+    """Queues of one width: the first factor of every group by its index (fewer
+    factors than groups, a last round with some), the rest from the counter."""
+    Gs, Js = _factors(n + 1, n, count)
+    a = api.hsvd_solve_batched(Gs, Js, api.make_batch_opts(group_width=1024))
+    for kw in (dict(), dict(group_width=512), dict(group_width=256), dict(cta_threads=512),
+               dict(group_width=256, cta_threads=512)):
+        assert _equal(a, api.hsvd_solve_batched(Gs, Js, api.make_batch_opts(**kw)), count)

@@ -45,11 +45,11 @@ METRIC = "HSVD time & eff. TFLOP/s at sigma rel-err <= 1e-12: new forms vs plain
 # kernel, from one ncu capture of this workload; an entry is removed when the
 # kernel changes
 PROFILED_TRAFFIC = {
-    ("graded1024", "fp64", "k_update<64>"): (17.317e6, "profiles/kernels_graded1024_fp64.md"),
-    ("graded1024", "fp64", "k_gram<32>"): (8.396e6, "profiles/kernels_graded1024_fp64.md"),
-    ("haar4096", "bf16x8", "k_update_x"): (498.15e6, "profiles/kernels_haar4096_bf16x8.md"),
-    ("haar4096", "bf16x8", "k_gram_x"): (151.58e6, "profiles/kernels_haar4096_bf16x8.md"),
-    ("haar4096", "bf16x8", "k_solve_cross<128,8>"): (18.97e6, "profiles/kernels_haar4096_bf16x8.md"),
+    ("graded1024", "fp64", "k_update<64>"): (17.318e6, "profiles/kernels_graded1024_fp64.md"),
+    ("graded1024", "fp64", "k_gram<32>"): (8.408e6, "profiles/kernels_graded1024_fp64.md"),
+    ("haar4096", "bf16x8", "k_update_x"): (498.37e6, "profiles/kernels_haar4096_bf16x8.md"),
+    ("haar4096", "bf16x8", "k_gram_x"): (151.02e6, "profiles/kernels_haar4096_bf16x8.md"),
+    ("haar4096", "bf16x8", "k_solve_cross<128,8>"): (18.975e6, "profiles/kernels_haar4096_bf16x8.md"),
 }
 # FP64 DFMA peak derived from the unit counts and the maximum clock (no FP64
 # figure in the measured peaks): 152 SMs x 2 DFMA/clk x 2 flop x 2070 MHz

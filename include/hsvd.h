@@ -384,10 +384,11 @@ int hsvd_sym_eig(const double *M, int64_t n, int64_t ldm, double *lambda, double
  * ones.  The group width of each size bucket (n < 40, < 72, < 128, < 192, and
  * larger) is picked by an autotuner that times the candidate widths on a
  * sample of the call's factors (two sweeps each) the first time a device sees
- * a set of buckets, and reuses that choice afterwards; in a short queue the
+ * a set of buckets, and reuses that choice afterwards (a bucket with fewer than
+ * four factors an SM is not timed and takes 256); in a short queue the
  * widths grow so that its largest factors do not outlast the rest.  A batch of
- * at most one factor per SM may run on one thread-block cluster per factor
- * instead (the same launch count, the same bits).
+ * at most one factor per SM may run on one thread-block cluster (of 1 to 16 CTAs)
+ * per factor instead (the same launch count, the same bits).
  */
 typedef struct hsvd_batch_opts {
     double tol;      /* <= 0: n_k 2^-53 for factor k                                */
@@ -407,9 +408,10 @@ typedef struct hsvd_batch_opts {
 typedef struct hsvd_batch_info {
     int grid;             /* CTAs of the launch (one per SM; a few factors: their
                              clusters' CTAs)                                        */
-    int tuned;            /* 1: the autotuner ran in this call, 2: its cached
-                             choice was used, 0: group_width was given or the
-                             factors were few enough for a cluster each             */
+    int tuned;            /* 1: this call chose the widths (by timing, for the
+                             buckets that fill the GPU: ms_tune, 0 if none does), 2: a
+                             choice of an earlier call was used, 0: group_width was
+                             given, or every factor ran on a cluster                */
     int bucket_width[5];  /* group width used per size bucket                      */
     int max_sweeps_run;   /* largest sweep count over the factors                  */
     int64_t rotations;    /* rotations applied, all factors                        */

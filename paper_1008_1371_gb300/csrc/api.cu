@@ -366,8 +366,8 @@ int solve_blocked_core(const double *G, int64_t m, int64_t n, int64_t ldg, const
     // GPU dispatches graph nodes at a bounded rate (about 2 us per node
     // measured), which would otherwise bound the sweep.  From n = 2048 a
     // visit's kernels take long enough for twice the nodes, smaller groups and
-    // more overlap (split precision: n = 2048 265 -> 261 ms; Haar 4096 1230 ms
-    // with a quarter of them, 1160 so, 1172 with twice as many).  Where a visit's
+    // more overlap (split precision: n = 2048 265 -> 261 ms; Haar 4096 1180 ms
+    // with a quarter of them, 1147 so).  Where a visit's
     // kernels are as short as their dispatch and a step's fill the chip, all of a
     // step goes into one group, and the capture costs a tenth (b = 16: n = 160
     // 7.9 -> 7.5 ms, 256 12.5 -> 11.1, 301 16.8 -> 15.1, 400 26.0 -> 24.5); up to
@@ -910,9 +910,10 @@ int hsvd_solve_ex(const double *G, int64_t m, int64_t n, int64_t ldg, const int8
         m > n && (o.shorten == HSVD_SHORTEN_ALWAYS || (o.shorten == HSVD_SHORTEN_AUTO && 4 * m >= 5 * n));
     const int64_t m_eff = shorten ? n : m;
     // the pointwise method below n = 32, the blocked one from there on.  On its
-    // cluster the pointwise kernel is the faster one up to n of about 150 now
-    // (n = 128: 5.95 against 8.5 ms), but the method fixes which value of sigma
-    // ends in which column, so the line stays where callers know it
+    // cluster the pointwise kernel is the faster one up to n of about 110 now
+    // (n = 64: 2.3 against 2.9 ms, 100: 4.6 and 5.2, 128: 5.7 and 5.3), but the
+    // method fixes which value of sigma ends in which column, so the line stays
+    // where callers know it
     int method = o.method;
     if (method == HSVD_METHOD_AUTO)
         method = (n < 32 && pointwise_fits(m_eff, n) && o.precision == HSVD_PRECISION_FP64) ? HSVD_METHOD_POINTWISE

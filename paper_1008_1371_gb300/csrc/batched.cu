@@ -397,8 +397,8 @@ std::map<long long, std::vector<int>> g_tune_cache;  // tune_key -> width per bu
 // scored by sum(m n^2) / time.  A bucket with fewer factors than the narrowest
 // width has groups cannot show what a full GPU does with it and is not timed:
 // it takes that width, the fastest per factor or within 1% of it wherever it
-// was measured (4000 factors of n in [16, 64]: 256: 46.9 ms, 512: 56.3, 1024:
-// 81.2; 2000 of [100, 140]: 413, 406, 437; 608 of 256: 846, 839, 862).
+// was measured (4000 factors of n in [16, 64]: 256: 46.6 ms, 512: 55.9, 1024:
+// 81.2; 2000 of [100, 140]: 390, 398, 426).
 // The choice is kept by device, CTA size, buckets present and buckets filled.
 long long tune_key(int dev, int cta, const std::vector<BTask> &all, int grid, int *filled) {
     int n[kBuckets] = {}, mask = 0;
@@ -466,9 +466,9 @@ cudaError_t tune_widths(const std::vector<BTask> &all, int grid, int cta, int *r
 // share of the work of this and the smaller buckets, which the queue holds
 // last; up to one warp for every four pairs (more only wait), and never below
 // a smaller bucket's width, so that the queue stays largest first.
-// Measured (n uniform on [16, 256], queue at 256 everywhere / at these widths
-// / on clusters): 600 factors 447 / 275 ms, 1000: 519 with the widths of n <
-// 128 left at 256 / 459, 40: 257 / 210 / 46, 100: 291 / 239 / 142.
+// Measured (n uniform on [16, 256], kernel, queue at 256 everywhere / at these
+// widths / on clusters): 600 factors 387 / 274 ms, 1000: 522 / 460, 300: 296 / 239,
+// 40: 247 / 207 / 46, 100: 286 / 239 / 142.
 void widen_for_tail(const std::vector<BTask> &tasks, int sms, int cta, std::vector<int> &width) {
     double sum[kBuckets] = {}, most[kBuckets] = {};
     for (const BTask &t : tasks) {

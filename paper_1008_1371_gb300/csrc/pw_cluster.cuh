@@ -38,8 +38,8 @@ __host__ __device__ inline size_t pw_cluster_smem(int64_t m_pad, int64_t n_pad, 
 // folded together), about 50 for the rotation, 4 (m + n) / 32 for the update.
 // Hence one pair per quarter of an SM's FP64 pipe: P <= 4 up to n = 128.
 // Measured (N(0,1), whole call, against the one-CTA kernel before it): n = 24:
-// 0.96 against 1.93 ms, n = 64: 2.39 against 13.2 ms, n = 128: 5.95 against
-// 52.5 ms (4.6 us a step, where one SM's FP64 rate made it 40 us).  The arithmetic is
+// 0.96 against 1.93 ms (0.84 with the scratch pool), n = 64: 2.39 against 13.2 ms,
+// n = 128: 5.7 against 52.5 ms (4.4 us a step, where one SM's FP64 rate made it 40 us).  The arithmetic is
 // pw_solve's, so the bits are those of the batched form.
 // out: status, sweeps, stop rule.
 static __device__ __forceinline__ void pw_cluster_solve(

@@ -227,12 +227,14 @@ cudaError_t cluster_config(int count, int C, const ClShape &s, cudaStream_t st, 
 // has a rotation of its own (56 instructions) and one barrier, 2,000.  0.8: the
 // later sweeps skip rotations and kept dots.  The clusters share the SMs' FP64
 // pipes, which no residency count shows (114 factors of n = 40: 3,200 cycles by
-// the longest factor, 17,000 by the pipes), at 250 cycles a CTA.  Clusters must be
-// estimated a fifth faster than groups; a smaller cluster must win 6 % (fewer
-// and fuller CTAs spread less evenly).  Measured, whole calls in ms, groups / this
-// choice: n = 8: 4 factors 0.53 / 0.40, 152 2.13 / 2.00; n = 16: 4 1.00 / 0.64, 152
-// 2.71 / 2.49; n = 40: 38 3.9 / 3.2, 114 4.6 / 4.6 (clusters of 16: 8.6); n = 64:
-// 38 7.2 / 4.5, 76 7.9 / 7.9 (8.5); n = 256: 38 220 / 150; 1024 x 8: 4 1.17 / 0.77.
+// the longest factor, 17,000 by the pipes), at 250 cycles a CTA and more where the
+// factors alone fill the SMs.  Clusters must be
+// estimated a quarter faster than groups, since they share the SMs less evenly than
+// the pipes' sum says; a smaller cluster must win 6 %.  Measured, the kernel in ms,
+// groups / this choice: n = 8: 4 factors 0.39 / 0.21, 152 0.40 / 0.23; n = 16: 4 0.76
+// / 0.45; n = 40: 38 3.3 / 2.6, 114 3.4 / 3.4 (clusters of 16: 7.2); n = 64: 38 6.6 /
+// 3.9, 76 6.9 / 6.9 (8.0); n = 256: 38 219 / 150; n from 10 to 70: 152 12.0 / 8.4, 114
+// 12.4 / 5.5; 16 to 128: 152 36 / 30; 1024 x 8: 4 0.96 / 0.56.
 int few_clusters(const std::vector<BTask> &tasks, const StreamLimits &limits, cudaStream_t st) {
     const int sms = limits.sms;
     if ((int)tasks.size() > sms) return 0;
@@ -241,12 +243,18 @@ int few_clusters(const std::vector<BTask> &tasks, const StreamLimits &limits, cu
     for (const BTask &t : tasks) {
         const double m = pw_rows_pad(t.m, t.n), n = t.n + (t.n & 1), half = n / 2;
         const double rows = 0.8 * (7.0 * m + 4.0 * n) / 32.0;
-        groups = std::max(groups, n * (std::max(half, 4.0) * rows * 16.0 + 10200.0));
+        // columns outside the group's shared memory: read from L2 twice a step
+        const int width = t.n < kBucketEdges[2] ? 256 : (t.n < kBucketEdges[3] ? 512 : 1024);
+        const double room = (double)kSmemBudget * width / 1024 - (double)pw_aux_bytes(t.n + (t.n & 1));
+        const double out = std::max(0.0, 1.0 - room / (double)need_bytes(t.m, t.n));
+        const double slow = width == 256 ? std::min(1.35, 1.0 + out) : 1.0 + 0.25 * out;
+        groups = std::max(groups, n * (std::max(half, 4.0) * rows * 16.0 * slow + 10200.0));
         pipes += n * half * (rows + 56.0) * 16.0;
         steps += n;
         most = std::max(most, (t.n + 1) / 2);
     }
-    const double line = 0.8 * groups;
+    const double line = 0.77 * groups;
+    const double per_cta = 250.0 * std::max(1.0, 2.0 * (double)tasks.size() / sms);
     double best = 0.0;
     int best_c = 0;
     for (int C : {16, 8, 4, 2, 1}) {
@@ -261,7 +269,7 @@ int few_clusters(const std::vector<BTask> &tasks, const StreamLimits &limits, cu
             c_sum += c;
         }
         const double bound = best_c ? std::min(line, 0.94 * best) : line;
-        double c = std::max(c_max, (pipes + 250.0 * C * steps) / sms);
+        double c = std::max(c_max, (pipes + per_cta * C * steps) / sms);
         if (c >= bound) continue;
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[1];
